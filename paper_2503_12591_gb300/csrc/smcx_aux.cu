@@ -99,6 +99,10 @@ void pair_counts_device(smcx_lattice* hd) {
     pair_counts_bcc_tiled(hd, nt);
     return;
   }
+  if (fcc_reduce_usable(hd, nt)) {
+    pair_counts_fcc_tiled(hd, nt);
+    return;
+  }
   const int K = hd->shells.K;
   if (hd->kind == kBCC) {
     switch (K) {

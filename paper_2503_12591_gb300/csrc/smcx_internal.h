@@ -175,6 +175,9 @@ void sweep_device(smcx_lattice* h, int nA, uint64_t seed, int64_t n_sweeps, int 
 bool bcc_fast_usable(const smcx_lattice* h, int dir_slots = 128);
 bool bcc_counts_usable(const smcx_lattice* h, int nt[3]);
 void pair_counts_bcc_tiled(smcx_lattice* h, const int nt[3]);
+bool fcc_reduce_usable(const smcx_lattice* h, int nt[3]);
+void pair_counts_fcc_tiled(smcx_lattice* h, const int nt[3]);
+bool qsro_energy_fcc_tiled(smcx_lattice* h);  // false if not applicable
 int bcc_slots_per_axis(const int n[3], const smcx_sched& sc);
 void bcc_block_shape(int nq, int tuned_threads, int* threads, int* slots);
 void sweep_bcc_fast(smcx_lattice* h, int nA, uint64_t seed, int64_t n_sweeps, int n_colours);

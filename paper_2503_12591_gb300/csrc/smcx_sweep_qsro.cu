@@ -1024,6 +1024,7 @@ void sweep_qsro_device(smcx_lattice* hd, int nA, uint64_t seed, int64_t n_sweeps
 }
 
 void qsro_energy_add(smcx_lattice* hd) {
+  if (qsro_energy_fcc_tiled(hd)) return;
   SweepParams P;
   memset(&P, 0, sizeof(P));
   P.sites = hd->d_sites;
