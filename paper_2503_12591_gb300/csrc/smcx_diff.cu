@@ -12,7 +12,7 @@
 // so an estimator needs sum(1), sum(A), sum(C), sum(A C^T) over samples; they
 // are accumulated on the device in FP64 (weighted, so that exact enumeration
 // can feed Boltzmann weights through the same code).
-#include "smcx_device.cuh"
+#include "smcx_fcc_tile.cuh"
 
 namespace smcx {
 
@@ -61,6 +61,179 @@ __global__ void __launch_bounds__(256) k_pair_counts_batch(const int8_t* __restr
     }
     __syncthreads();
     for (int i = threadIdx.x; i < KMM; i += blockDim.x) out[b * KMM + i] = bad ? -1ll : (long long)hist[i];
+    __syncthreads();
+  }
+}
+
+// Half-shell vectors of a lattice kind, and where they lead from site b of a cell:
+// (dx, dy, dz) cells and the site there, fixed at compile time.
+struct HalfVec {
+  signed char dx, dy, dz, b, k;
+};
+struct HalfVecs {
+  HalfVec v[4][25];
+  int n;
+};
+__host__ __device__ constexpr int floor_half(int p) { return p >= 0 ? p / 2 : -((1 - p) / 2); }
+template <int KIND, int K>
+__host__ __device__ constexpr HalfVecs make_half_vecs() {
+  HalfVecs H{};
+  constexpr int basis[2][4][3] = {{{0, 0, 0}, {1, 1, 1}, {0, 0, 0}, {0, 0, 0}}, {{0, 0, 0}, {1, 1, 0}, {1, 0, 1}, {0, 1, 1}}};
+  H.n = 0;
+  for (int x = 0; x <= 3; x++)
+    for (int y = -3; y <= 3; y++)
+      for (int z = -3; z <= 3; z++) {
+        if (!(x > 0 || (x == 0 && (y > 0 || (y == 0 && z > 0))))) continue;
+        int k = -1;
+        if (KIND == kBCC) {
+          const bool same = ((x ^ y) & 1) == 0 && ((x ^ z) & 1) == 0;
+          k = same ? bccfast::bcc_shell_of(x, y, z) : -1;
+        } else if (((x + y + z) & 1) == 0) {
+          const int r = x * x + y * y + z * z;
+          k = r == 2 ? 0 : r == 4 ? 1 : r == 6 ? 2 : -1;
+        }
+        if (k < 0 || k >= K) continue;
+        for (int b = 0; b < cell_sites(KIND); b++) {
+          const int px = basis[KIND == kFCC][b][0] + x, py = basis[KIND == kFCC][b][1] + y, pz = basis[KIND == kFCC][b][2] + z;
+          HalfVec& h = H.v[b][H.n];
+          h.dx = (signed char)floor_half(px);
+          h.dy = (signed char)floor_half(py);
+          h.dz = (signed char)floor_half(pz);
+          for (int t = 0; t < cell_sites(KIND); t++)
+            if (basis[KIND == kFCC][t][0] == (px & 1) && basis[KIND == kFCC][t][1] == (py & 1) &&
+                basis[KIND == kFCC][t][2] == (pz & 1))
+              h.b = (signed char)t;
+          h.k = (signed char)k;
+        }
+        H.n++;
+      }
+  return H;
+}
+
+// Pair counts for at most 4 W species (W = 1 or 2 counter words): one CTA per
+// configuration, staged as 8 s in shared memory; a thread takes whole cells.
+// Every unordered pair once: a neighbour of the half shell k adds 1 << (8 s) to
+// byte counters (at most 12), which are added to the counters of the centre's
+// species, C[p][q] = U[p][q] + U[q][p].  A thread empties its byte counters
+// after 20 sites at most (20 x 12 < 256).  Bound by issue; 4096 configurations of
+// 1,024 sites take 54 us against 215 for k_pair_counts_batch, which makes one
+// shared atomic per neighbour over whole shells (50 a site) and stays for more
+// than eight species and for edges of one cell.
+template <int KIND, int K, int W>
+__global__ void __launch_bounds__(256) k_pair_counts_batch_half(const int8_t* __restrict__ cfg, long long B, int nx,
+                                                                int ny, int nz, int M, long long* __restrict__ out) {
+  constexpr int m = cell_sites(KIND);
+  constexpr HalfVecs H = make_half_vecs<KIND, K>();
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ unsigned hist[K * 64];
+  uint8_t* s = smem;
+  const int ncell = nx * ny * nz, N = ncell * m, KMM = K * M * M;
+  const int lane = threadIdx.x & 31;
+  for (long long b = blockIdx.x; b < B; b += gridDim.x) {
+    for (int i = threadIdx.x; i < K * 64; i += blockDim.x) hist[i] = 0;
+    const int8_t* c = cfg + b * N;
+    int bad = 0;
+    if ((reinterpret_cast<uintptr_t>(c) & 3) == 0) {  // N is even: whole words up to a tail of 2
+      const uint32_t* cw = reinterpret_cast<const uint32_t*>(c);
+      for (int i = threadIdx.x; i < N / 4; i += blockDim.x) {
+        const uint32_t v = cw[i];
+#pragma unroll
+        for (int j = 0; j < 4; j++) bad |= (int)((v >> (8 * j)) & 255u) >= M;
+        reinterpret_cast<uint32_t*>(s)[i] = (v & 0x1F1F1F1Fu) << 3;
+      }
+      for (int i = N / 4 * 4 + threadIdx.x; i < N; i += blockDim.x) {
+        bad |= (uint8_t)c[i] >= M;
+        s[i] = (uint8_t)((c[i] & 31) << 3);
+      }
+    } else {
+      for (int i = threadIdx.x; i < N; i += blockDim.x) {
+        bad |= (uint8_t)c[i] >= M;
+        s[i] = (uint8_t)((c[i] & 31) << 3);
+      }
+    }
+    // a configuration holding an id outside 0..M-1 is not counted; all its
+    // counts are set to -1
+    bad = __syncthreads_or(bad);
+    uint32_t acc[K][4 * W][W];
+    auto clear = [&]() {
+#pragma unroll
+      for (int k = 0; k < K; k++)
+#pragma unroll
+        for (int p = 0; p < 4 * W; p++)
+#pragma unroll
+          for (int w = 0; w < W; w++) acc[k][p][w] = 0;
+    };
+    // byte counters of the warp's threads into the histogram; called by whole warps
+    auto flush = [&]() {
+#pragma unroll
+      for (int k = 0; k < K; k++)
+#pragma unroll
+        for (int p = 0; p < 4 * W; p++)
+#pragma unroll
+          for (int w = 0; w < W; w++) {
+            const uint32_t e = __reduce_add_sync(0xffffffffu, acc[k][p][w] & 0x00FF00FFu);
+            const uint32_t o = __reduce_add_sync(0xffffffffu, (acc[k][p][w] >> 8) & 0x00FF00FFu);
+            // lane q < 4 adds species 4 w + q
+            const uint32_t v = (((lane & 1) ? o : e) >> (lane & 2 ? 16 : 0)) & 0xFFFFu;
+            if (lane < 4 && v) atomicAdd(&hist[k * 64 + p * 8 + 4 * w + lane], v);
+          }
+      clear();
+    };
+    clear();
+    int held = 0;
+    for (int c0 = 0; !bad && c0 < ncell; c0 += blockDim.x) {
+      const int cell = c0 + threadIdx.x;
+      if (cell < ncell) {
+        const int x = cell % nx, r = cell / nx, y = r % ny, z = r / ny;
+        int ox[5], oy[5], oz[5];  // byte offsets of displacements -2 .. 2
+#pragma unroll
+        for (int d = -2; d <= 2; d++) {
+          ox[d + 2] = wrap_add(x, d, nx) * m;
+          oy[d + 2] = wrap_add(y, d, ny) * nx * m;
+          oz[d + 2] = wrap_add(z, d, nz) * ny * nx * m;
+        }
+#pragma unroll
+        for (int bs = 0; bs < m; bs++) {
+          const int p8 = s[cell * m + bs];
+          uint32_t h[K][W];
+#pragma unroll
+          for (int k = 0; k < K; k++)
+#pragma unroll
+            for (int w = 0; w < W; w++) h[k][w] = 0;
+#pragma unroll
+          for (int j = 0; j < H.n; j++) {
+            const HalfVec v = H.v[bs][j];
+            const uint32_t q8 = s[(oz[v.dz + 2] + oy[v.dy + 2]) + ox[v.dx + 2] + v.b];
+            uint32_t lo, hi;
+            asm("shl.b32 %0, 1, %1;" : "=r"(lo) : "r"(q8));
+            h[v.k][0] += lo;
+            if (W == 2) {
+              asm("shl.b32 %0, 1, %1;" : "=r"(hi) : "r"(q8 - 32u));
+              h[v.k][W - 1] += hi;
+            }
+          }
+#pragma unroll
+          for (int p = 0; p < 4 * W; p++) {
+            if (p8 != 8 * p) continue;
+#pragma unroll
+            for (int k = 0; k < K; k++)
+#pragma unroll
+              for (int w = 0; w < W; w++) acc[k][p][w] += h[k][w];
+          }
+        }
+      }
+      held += m;
+      if (held + m > 20) {
+        flush();
+        held = 0;
+      }
+    }
+    if (held) flush();
+    __syncthreads();
+    for (int i = threadIdx.x; i < KMM; i += blockDim.x) {
+      const int k = i / (M * M), p = (i / M) % M, q = i % M;
+      out[b * KMM + i] = bad ? -1ll : (long long)hist[k * 64 + p * 8 + q] + (long long)hist[k * 64 + q * 8 + p];
+    }
     __syncthreads();
   }
 }
@@ -218,11 +391,38 @@ int smcx_pair_counts_batch(int kind, int nx, int ny, int nz, int M, int K, const
     const size_t smem = (size_t)KMM * 4 + (size_t)N;
     if (smem > 200 * 1024) fail(SMCX_E_UNSUPPORTED, "configurations above ~200k sites: use smcx_pair_counts");
     if (B == 0) return;
+    cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+    const int grid = (int)std::min<long long>(B, 65535);
+    // at most eight species: counted in registers over half shells (edges of the
+    // reach of 2 cells at least, so that one wrap covers every displacement)
+    if (M <= 8 && nx >= 2 && ny >= 2 && nz >= 2) {
+      const int ncell = nx * ny * nz;
+      const int threads = std::min(256, (ncell + 31) / 32 * 32);
+      const size_t sm = (size_t)(N + 3) / 4 * 4;
+      auto run = [&](auto kern) {
+        check_cuda(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm), "smem attr");
+        kern<<<grid, threads, sm, st>>>(d_configs, B, nx, ny, nz, M, reinterpret_cast<long long*>(d_counts));
+      };
+      auto pick = [&](auto k4, auto k8) {
+        if (M <= 4) run(k4);
+        else run(k8);
+      };
+      if (kind == kBCC) {
+        if (K == 1) pick(k_pair_counts_batch_half<kBCC, 1, 1>, k_pair_counts_batch_half<kBCC, 1, 2>);
+        else if (K == 2) pick(k_pair_counts_batch_half<kBCC, 2, 1>, k_pair_counts_batch_half<kBCC, 2, 2>);
+        else if (K == 3) pick(k_pair_counts_batch_half<kBCC, 3, 1>, k_pair_counts_batch_half<kBCC, 3, 2>);
+        else pick(k_pair_counts_batch_half<kBCC, 4, 1>, k_pair_counts_batch_half<kBCC, 4, 2>);
+      } else {
+        if (K == 1) pick(k_pair_counts_batch_half<kFCC, 1, 1>, k_pair_counts_batch_half<kFCC, 1, 2>);
+        else if (K == 2) pick(k_pair_counts_batch_half<kFCC, 2, 1>, k_pair_counts_batch_half<kFCC, 2, 2>);
+        else pick(k_pair_counts_batch_half<kFCC, 3, 1>, k_pair_counts_batch_half<kFCC, 3, 2>);
+      }
+      check_cuda(cudaGetLastError(), "pair-count batch launch");
+      return;
+    }
     SweepParams P;
     memset(&P, 0, sizeof(P));
     fill_offsets_kind(kind, S, P);
-    cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    const int grid = (int)std::min<long long>(B, 65535);
     auto go = [&](auto kern) {
       check_cuda(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem), "smem attr");
       kern<<<grid, 256, smem, st>>>(d_configs, B, nx, ny, nz, M, P, reinterpret_cast<long long*>(d_counts));

@@ -62,13 +62,10 @@ void check_reach(const Shells& S, const int n[3]) {
   }
 }
 
-Shells make_shells(int kind, int K) {
+static Shells build_shells(int kind, int K) {
   Shells s;
   s.kind = kind;
   s.m = sites_per_cell(kind);
-  if (s.m == 0) fail(SMCX_E_INVALID_ARG, "unknown lattice kind");
-  int kmax = kind == kBCC ? 4 : 3;
-  if (K < 1 || K > kmax) fail(SMCX_E_INVALID_ARG, "shell count out of range for this lattice");
   // every lattice vector within 3 cells, keyed by (|v|^2, vx, vy, vz)
   std::vector<std::array<int, 4>> all;
   for (int cx = -3; cx <= 3; cx++)
@@ -104,6 +101,21 @@ Shells make_shells(int kind, int K) {
       if (s.shell_of[i] == 0) s.R1 = std::max(s.R1, a);
     }
   return s;
+}
+
+// The shells depend on the lattice kind and K alone: built once per process (the
+// sort of the vectors took longer than a small launch).
+Shells make_shells(int kind, int K) {
+  if (sites_per_cell(kind) == 0) fail(SMCX_E_INVALID_ARG, "unknown lattice kind");
+  const int kmax = kind == kBCC ? 4 : 3;
+  if (K < 1 || K > kmax) fail(SMCX_E_INVALID_ARG, "shell count out of range for this lattice");
+  static const std::array<std::array<Shells, kMaxShells>, 2> table = [] {
+    std::array<std::array<Shells, kMaxShells>, 2> t;
+    for (int k = 1; k <= 4; k++) t[0][k - 1] = build_shells(kBCC, k);
+    for (int k = 1; k <= 3; k++) t[1][k - 1] = build_shells(kFCC, k);
+    return t;
+  }();
+  return table[kind == kBCC ? 0 : 1][K - 1];
 }
 
 // Two trials whose centres are 2L half-units apart on one axis cannot touch

@@ -1,11 +1,11 @@
-"""Tiled reductions against the oracle at
+"""Tiled reductions and batched pair counts against the oracle at
 the sizes where they can go wrong: tile edges and remainders, tiles that wrap
 onto themselves, the most species, counters emptied between sites."""
 import numpy as np
 import pytest
 
 import oracle as O
-from paper_2503_12591_gb300 import smcx
+from paper_2503_12591_gb300 import diff, smcx
 from paper_2503_12591_gb300.inputs import epi_gaussian
 
 pytestmark = pytest.mark.gpu
@@ -40,3 +40,20 @@ def test_fcc_counts_and_energies(dims, M, K, storage):
             return  # no schedule for the longer reach: the model is refused
         assert lat.energy() == O.energy_qsro(O.FCC, dims, M, K, V, W, cfg)
     lat.close()
+
+
+@pytest.mark.parametrize("kind,dims,M,K,B", [
+    (smcx.BCC, (2, 2, 2), 4, 4, 3), (smcx.BCC, (3, 5, 7), 8, 4, 5), (smcx.BCC, (14, 15, 16), 4, 3, 3),
+    (smcx.BCC, (5, 4, 3), 5, 1, 9), (smcx.BCC, (9, 9, 9), 1, 2, 2), (smcx.FCC, (2, 2, 3), 7, 3, 4),
+    (smcx.FCC, (12, 13, 11), 5, 3, 3), (smcx.FCC, (3, 3, 3), 4, 2, 11), (smcx.FCC, (1, 2, 2), 3, 1, 4),
+    (smcx.BCC, (8, 8, 8), 9, 4, 3)])
+def test_pair_counts_batch_sizes(kind, dims, M, K, B):
+    N = O.n_sites(kind, dims)
+    cfg = np.random.default_rng(11).integers(0, M, (B, N)).astype(np.int8)
+    pad = torch.zeros(B * N + 3, dtype=torch.int8, device="cuda")
+    for off in (0, 2):  # whole words of a configuration, and not
+        view = pad[off:off + B * N]
+        view.copy_(torch.from_numpy(cfg.reshape(-1)))
+        C = diff.pair_counts(view.view(B, N), kind, dims, M, K).cpu().numpy()
+        for b in range(B):
+            assert (C[b] == O.pair_counts(kind, dims, M, K, cfg[b])).all()
