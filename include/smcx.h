@@ -328,13 +328,15 @@ int smcx_sro(smcx_lattice* h, double* alpha);
  *   one class are in one cluster.  d_labels (device, [N] int32, caller-owned)
  *   receives for every site the smallest site id of its cluster (a unique
  *   labelling); *n_clusters (may be NULL) the number of clusters.  Needs N <
- *   2^31 (SMCX_E_RANGE); temporary device memory N bytes.  SMCX_E_TIMEOUT if
+ *   2^31 (SMCX_E_RANGE); device scratch of N bytes.  SMCX_E_TIMEOUT if
  *   the union-find exceeded its iteration limit (labels then undefined).
  * smcx_cluster_summary: from labels made by smcx_clusters on this handle's
  *   current configuration, the clusters of at least min_size sites, largest
  *   first (ties: smaller label first), at most max_out of them: roots [max_out]
  *   (labels), sizes [max_out], counts [max_out][M] (species counts, may be
- *   NULL); *n_out = number written.  Temporary device memory 4 N bytes.
+ *   NULL); *n_out = number written.  Device scratch of 4 N bytes and a list of
+ *   up to 2^20 clusters.  Scratch of up to 256 MiB stays with the handle until
+ *   smcx_lattice_destroy; more is released with the call.
  *   SMCX_E_RANGE if more than 2^26 clusters reach min_size.
  */
 int smcx_local_energy(smcx_lattice* h, int32_t* d_e2);

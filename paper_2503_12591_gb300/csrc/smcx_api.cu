@@ -48,6 +48,7 @@ void release(smcx_lattice* h) {
   cudaFree(h->d_flag);
   cudaFree(h->d_stage);
   cudaFree(h->d_qcnt);
+  cudaFree(h->d_scratch);
 }
 
 // One int8 id per site, allocated on first configuration transfer and kept.

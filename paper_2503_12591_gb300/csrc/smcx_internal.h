@@ -136,6 +136,8 @@ struct smcx_lattice {
   uint8_t* d_stage = nullptr;             // host<->device staging (int8 ids)
   uint16_t* d_qcnt = nullptr;             // qSRO same-species counts, one word per site (FCC sweeps)
   size_t stage_bytes = 0;
+  uint8_t* d_scratch = nullptr;           // kept scratch of the cluster calls (bounded, smcx_cluster.cu)
+  size_t scratch_bytes = 0;
 
   int kernel_choice = 0;  // 0 = fastest usable, 1 = generic tile/link-cell kernels
   int replica = 0;        // Philox replica id (counter word 1, bits 16..31)

@@ -1,4 +1,4 @@
-"""Tiled reductions and batched pair counts against the oracle at
+"""Tiled reductions, tiled clusters and batched pair counts against the oracle at
 the sizes where they can go wrong: tile edges and remainders, tiles that wrap
 onto themselves, the most species, counters emptied between sites."""
 import numpy as np
@@ -39,6 +39,42 @@ def test_fcc_counts_and_energies(dims, M, K, storage):
         except smcx.SmcxError:
             return  # no schedule for the longer reach: the model is refused
         assert lat.energy() == O.energy_qsro(O.FCC, dims, M, K, V, W, cfg)
+    lat.close()
+
+
+@pytest.mark.parametrize("kind,dims,M,K,storage", [
+    (smcx.FCC, (2, 3, 2), 4, 3, smcx.INT8), (smcx.FCC, (25, 13, 26), 5, 3, smcx.PACKED4),
+    (smcx.FCC, (13, 12, 37), 8, 2, smcx.INT8), (smcx.FCC, (50, 49, 4), 3, 1, smcx.PACKED4),
+    (smcx.BCC, (4, 3, 5), 4, 2, smcx.INT8), (smcx.BCC, (33, 17, 20), 4, 4, smcx.PACKED4),
+    (smcx.BCC, (16, 49, 9), 3, 3, smcx.INT8), (smcx.BCC, (21, 10, 8), 6, 4, smcx.INT8)])
+@pytest.mark.parametrize("qsro", [False, True])
+def test_clusters_in_tiles(kind, dims, M, K, storage, qsro):
+    lat, cfg, V = _lattice(kind, dims, M, K, storage, 5)
+    W = np.random.default_rng(8).integers(-60, 61, (K, M)).astype(np.int32)
+    if qsro:
+        try:
+            lat.set_qsro(W)
+        except smcx.SmcxError as e:
+            pytest.skip(f"schedule: {e}")
+    N = cfg.size
+    e2 = torch.empty(N, dtype=torch.int32, device="cuda")
+    lat.local_energy(e2.data_ptr())
+    lat.synchronize()
+    want = (O.local_energy2_qsro(kind, dims, M, K, V, W, cfg) if qsro else O.local_energy2(kind, dims, M, K, V, cfg))
+    assert (e2.cpu().numpy() == want).all()
+    lab = torch.empty(N, dtype=torch.int32, device="cuda")
+    for q in (0.0, 0.2, 0.5, 0.85, 1.0):
+        thr = int(np.quantile(want, q))
+        n = lat.clusters(thr, lab.data_ptr())
+        ref, rn = (O.clusters_qsro(kind, dims, M, K, V, W, cfg, thr) if qsro
+                   else O.clusters(kind, dims, M, K, V, cfg, thr))
+        assert n == rn and (lab.cpu().numpy() == ref).all()
+        for min_size, most in ((1, 3000), (3, 7)):
+            roots, sizes, counts = lat.cluster_summary(lab.data_ptr(), min_size, most)
+            oroots, osizes, ocounts = O.cluster_summary(ref, cfg, M, min_size)
+            k = min(most, oroots.size)
+            assert roots.tolist() == oroots[:k].tolist() and sizes.tolist() == osizes[:k].tolist()
+            assert counts.tolist() == ocounts[:k].tolist()
     lat.close()
 
 
