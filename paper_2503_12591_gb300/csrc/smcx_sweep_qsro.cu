@@ -559,7 +559,7 @@ __device__ __forceinline__ int pair_side(const uint16_t* box, int e, const int32
 // in the even-point box, n_k(i) counted there, one 16-bit
 // word per site (n_0 | n_1 << 4 | n_2 << 7) written to cnt[4 cell + b].
 template <int K>
-__global__ void __launch_bounds__(128) k_qsro_fcc_count_init(const SweepParams P, uint16_t* __restrict__ cnt) {
+__global__ void __launch_bounds__(512) k_qsro_fcc_count_init(const SweepParams P, uint16_t* __restrict__ cnt) {
   using namespace qfcc;
   extern __shared__ __align__(16) unsigned char smem[];
   uint8_t* box = smem;
@@ -588,167 +588,82 @@ __global__ void __launch_bounds__(128) k_qsro_fcc_count_init(const SweepParams P
   }
 }
 
-template <int K, int TM>
-__global__ void __launch_bounds__(128, TM == 20 ? 2 : 3)
-    k_qsro_fcc_n(const SweepParams P, const QsroTables Q, uint16_t* __restrict__ cnt) {
-  using namespace qfn;
-  using BX = QBox<TM>;
-  constexpr int BOX_BYTES = BX::BOX_BYTES;
-  constexpr qfcc::QTable T = qfcc::make_qvecs();
-  constexpr int NV = vec_count(kFCC, K);
-  extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ unsigned long long s_stat[3];
-  __shared__ int32_t s_wq[kMaxShells * kMaxSweepM];
-  constexpr QClass<K> QC = make_qclass<K, TM>();
-  constexpr int NS = QC.NS, NP = QC.NP;
-  __shared__ short s_es[12 * NS], s_ep[12 * NP];
-  __shared__ int s_qoff[NV];
-
-  const int tid = threadIdx.x, nth = blockDim.x;
-  const int lane = tid & 31, warp = tid >> 5, nwarp = nth >> 5;
-  const int M = P.M, KM = K * P.M, MM = P.M * P.M;
-  const int nW = MM * KM + MM;
-  uint16_t* box = reinterpret_cast<uint16_t*>(smem);
-  int32_t* s_w = reinterpret_cast<int32_t*>(smem + BOX_BYTES);
-
+namespace qfn {
+// Tile of this CTA among the tiles of colour P.tc.
+__device__ __forceinline__ void colour_tile(const SweepParams& P, int (&t0)[3], int (&ts)[3]) {
   int bid = blockIdx.x;
   const int jx = bid % P.ntc[0];
   bid /= P.ntc[0];
   const int jy = bid % P.ntc[1];
   const int jz = bid / P.ntc[1];
   const int ti[3] = {2 * jx + (P.tc & 1), 2 * jy + ((P.tc >> 1) & 1), 2 * jz + ((P.tc >> 2) & 1)};
-  int t0[3], ts[3];
 #pragma unroll
   for (int a = 0; a < 3; a++) {
     const int base = P.n[a] / P.nt[a], rem = P.n[a] % P.nt[a];
     ts[a] = base + (ti[a] < rem ? 1 : 0);
     t0[a] = ti[a] * base + min(ti[a], rem);
   }
-  if (tid < 3) s_stat[tid] = 0;
-  for (int i = tid; i < nW; i += nth) s_w[i] = P.wtab[i];
-  for (int i = tid; i < KM; i += nth) s_wq[i] = Q.W[i];
-  for (int i = tid; i < 12 * NS; i += nth) s_es[i] = (qclass<K, TM>().es)[i / NS][i % NS];
-  for (int i = tid; i < 12 * NP; i += nth) s_ep[i] = (qclass<K, TM>().ep)[i / NP][i % NP];
-  if (tid < NV) {
-    int o = 0;
-#pragma unroll
-    for (int j = 0; j < NV; j++)
-      if (j == tid) o = BX::voff(T.v[j].x, T.v[j].y, T.v[j].z);
-    s_qoff[tid] = o;  // the first 12 entries are the partner offsets
-  }
+}
 
-  // stage the cells [t0 - 2, t0 + ts + 2) of each axis: species and counts,
-  // the sites inside the box (box coordinate 2 i - 1 + basis in [0, 2 ts + 5])
+// Stage the cells [t0 - 2, t0 + ts + 2) of each axis: species and counts, the
+// sites inside the box (box coordinate 2 i - 1 + basis in [0, 2 ts + 5]).  One box
+// column per lane (ex <= 24 < 32), warp w the planes w, w + nwarp, ..., the loads
+// of U rows of a plane issued before any is unpacked.
+template <int TM>
+__device__ __forceinline__ void stage(const SweepParams& P, const uint16_t* cnt, uint16_t* box, const int (&t0)[3],
+                                      const int (&ts)[3]) {
+  using BX = QBox<TM>;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
   const int nx = P.n[0], ny = P.n[1], nz = P.n[2];
   const int ex = ts[0] + 4, ey = ts[1] + 4, ez = ts[2] + 4;
   const int lim[3] = {2 * ts[0] + 5, 2 * ts[1] + 5, 2 * ts[2] + 5};
-  {
-    // one box column per lane (ex <= 24 < 32), warp w the planes w, w +
-    // nwarp, ..., the loads of U rows of a plane issued before any is
-    // unpacked
-    constexpr int U = 8;
-    const int gx = lane < ex ? wrap_add(t0[0] - 2, lane, nx) : 0;
-    for (int zs = warp; zs < ez; zs += nwarp) {
-      const long long zrow = (long long)wrap_add(t0[2] - 2, zs, nz) * ny;
-      for (int ys0 = 0; ys0 < ey; ys0 += U) {
-        uint32_t v[U];
-        uint2 c4[U];
+  constexpr int U = 8;
+  const int gx = lane < ex ? wrap_add(t0[0] - 2, lane, nx) : 0;
+  for (int zs = warp; zs < ez; zs += nwarp) {
+    const long long zrow = (long long)wrap_add(t0[2] - 2, zs, nz) * ny;
+    for (int ys0 = 0; ys0 < ey; ys0 += U) {
+      uint32_t v[U];
+      uint2 c4[U];
 #pragma unroll
-        for (int u = 0; u < U; u++) {
-          const int ys = ys0 + u;
-          v[u] = 0;
-          c4[u] = make_uint2(0, 0);
-          if (ys < ey && lane < ex) {
-            const long long cell = (zrow + wrap_add(t0[1] - 2, ys, ny)) * nx + gx;
-            v[u] = P.storage == SMCX_INT8 ? *reinterpret_cast<const uint32_t*>(P.sites + 4 * cell)
-                                          : (uint32_t)(*reinterpret_cast<const uint16_t*>(P.sites + 2 * cell));
-            c4[u] = *reinterpret_cast<const uint2*>(cnt + 4 * cell);
-          }
+      for (int u = 0; u < U; u++) {
+        const int ys = ys0 + u;
+        v[u] = 0;
+        c4[u] = make_uint2(0, 0);
+        if (ys < ey && lane < ex) {
+          const long long cell = (zrow + wrap_add(t0[1] - 2, ys, ny)) * nx + gx;
+          v[u] = P.storage == SMCX_INT8 ? *reinterpret_cast<const uint32_t*>(P.sites + 4 * cell)
+                                        : (uint32_t)(*reinterpret_cast<const uint16_t*>(P.sites + 2 * cell));
+          c4[u] = *reinterpret_cast<const uint2*>(cnt + 4 * cell);
         }
+      }
 #pragma unroll
-        for (int u = 0; u < U; u++) {
-          const int ys = ys0 + u;
-          if (ys < ey && lane < ex) {
+      for (int u = 0; u < U; u++) {
+        const int ys = ys0 + u;
+        if (ys < ey && lane < ex) {
 #pragma unroll
-            for (int b = 0; b < 4; b++) {
-              const int x = 2 * lane - 1 + bx_of(b), y = 2 * ys - 1 + by_of(b), z = 2 * zs - 1 + bz_of(b);
-              if (x < 0 || y < 0 || z < 0 || x > lim[0] || y > lim[1] || z > lim[2]) continue;
-              const uint32_t sp = P.storage == SMCX_INT8 ? (v[u] >> (8 * b)) & 0xFFu : (v[u] >> (4 * b)) & 15u;
-              const uint32_t cw = ((b < 2 ? c4[u].x : c4[u].y) >> (16 * (b & 1))) & 0xFFFFu;
-              box[BX::eidx(x, y, z)] = (uint16_t)(sp | (cw << 3));
-            }
+          for (int b = 0; b < 4; b++) {
+            const int x = 2 * lane - 1 + bx_of(b), y = 2 * ys - 1 + by_of(b), z = 2 * zs - 1 + bz_of(b);
+            if (x < 0 || y < 0 || z < 0 || x > lim[0] || y > lim[1] || z > lim[2]) continue;
+            const uint32_t sp = P.storage == SMCX_INT8 ? (v[u] >> (8 * b)) & 0xFFu : (v[u] >> (4 * b)) & 15u;
+            const uint32_t cw = ((b < 2 ? c4[u].x : c4[u].y) >> (16 * (b & 1))) & 0xFFFFu;
+            box[BX::eidx(x, y, z)] = (uint16_t)(sp | (cw << 3));
           }
         }
       }
     }
   }
-  __syncthreads();
+}
 
-  unsigned long long acc = 0, same = 0;
-  long long dsum = 0;
-  const int L = P.L;
-  const int NQ = (max(ts[0], max(ts[1], ts[2])) + L - 1) / L;
-  const int qx = tid % NQ, qy = (tid / NQ) % NQ, qz = tid / (NQ * NQ);
-  const bool slot = tid < NQ * NQ * NQ;
-  for (int cz = 0; cz < L; cz++)
-    for (int cy = 0; cy < L; cy++)
-      for (int cx = 0; cx < L; cx++) {
-        const int xr = cx + L * qx, yr = cy + L * qy, zr = cz + L * qz;
-        const bool here = slot && xr < ts[0] && yr < ts[1] && zr < ts[2];
-        const int cbase = BX::eidx(2 * xr + 3, 2 * yr + 3, 2 * zr + 3);
-        const unsigned long long cell = ((unsigned long long)(t0[2] + zr) * ny + (t0[1] + yr)) * nx + (t0[0] + xr);
-        uint4 rw = make_uint4(0, 0, 0, 0);
-        for (int b = 0; b < 4; b++) {
-          if (here) {
-            if ((b & 1) == 0) rw = attempt_block(cell * 4 + b, P.sweep, P.replica, P.seed_lo, P.seed_hi);
-            const uint32_t rd = (b & 1) ? rw.z : rw.x;
-            const uint32_t ru = (b & 1) ? rw.w : rw.y;
-            const int s = cbase + BX::voff(bx_of(b), by_of(b), bz_of(b));
-            const int dir = (int)__umulhi(rd, 12u);
-            const int sp = s + s_qoff[dir];
-            const int sa = box[s] & 7, sb = box[sp] & 7;
-            if (sa == sb) {
-              same++;
-            } else {
-              const int32_t* W = s_w + (sa * M + sb) * KM;
-              int wqa[K], wqb[K];
-#pragma unroll
-              for (int k = 0; k < K; k++) {
-                wqa[k] = s_wq[k * M + sa];
-                wqb[k] = s_wq[k * M + sb];
-              }
-              // pair part and the counts of s and s' after the swap: b
-              // around s without s' (which holds b before the swap), a around
-              // s' without s
-              int na_s[K], nb_s[K], na_p[K], nb_p[K];
-              int dE = s_w[MM * KM + sa * M + sb] + pair_side<K, TM, 1>(box, s, W, M, sa, sb, na_s, nb_s) +
-                       pair_side<K, TM, -1>(box, sp, W, M, sa, sb, na_p, nb_p);
-              nb_s[0]--;
-              na_p[0]--;
-#pragma unroll
-              for (int k = 0; k < K; k++)
-                dE += wqb[k] * (nb_s[k] * nb_s[k] - nb_p[k] * nb_p[k]) + wqa[k] * (na_p[k] * na_p[k] - na_s[k] * na_s[k]);
-              // environment sites whose counts move
-              const short* es = s_es + dir * NS;
-              const short* ep = s_ep + dir * NP;
-              dE += es_energy<K, TM, 0, NS>(box, es, s, sa, sb, wqa, wqb);
-              dE += ep_energy<K, TM>(box, ep, sp, sa, sb, wqa, wqb);
-              if (metropolis_accept(dE, ru, P.thr, P.nA, P.thr + kNA)) {
-                box[s] = (uint16_t)(sb | (pack_counts<K>(nb_s) << 3));
-                box[sp] = (uint16_t)(sa | (pack_counts<K>(na_p) << 3));
-                es_update<K, TM, 0, NS>(box, es, s, sa, sb);
-                ep_update<K, TM>(box, ep, sp, sa, sb);
-                acc++;
-                dsum += dE;
-              }
-            }
-          }
-          __syncthreads();
-        }
-      }
-
-  // write back the species of the tile and its 1-cell ring, the counts of
-  // every site in the box
+// Write back the species of the tile and its 1-cell ring, the counts of every site
+// in the box.
+template <int TM>
+__device__ __forceinline__ void write_back(const SweepParams& P, uint16_t* cnt, const uint16_t* box, const int (&t0)[3],
+                                           const int (&ts)[3]) {
+  using BX = QBox<TM>;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
+  const int nx = P.n[0], ny = P.n[1], nz = P.n[2];
+  const int ex = ts[0] + 4, ey = ts[1] + 4, ez = ts[2] + 4;
+  const int lim[3] = {2 * ts[0] + 5, 2 * ts[1] + 5, 2 * ts[2] + 5};
   const int gxs = lane < ex ? wrap_add(t0[0] - 2, lane, nx) : 0;
   for (int zs = warp; zs < ez; zs += nwarp) {
     const long long zrow = (long long)wrap_add(t0[2] - 2, zs, nz) * ny;
@@ -785,14 +700,281 @@ __global__ void __launch_bounds__(128, TM == 20 ? 2 : 3)
       }
     }
   }
-  add_stats_warp(s_stat, (unsigned)acc, (unsigned)same, dsum);
-  __syncthreads();
-  if (tid == 0) {
-    atomicAdd(&P.stats[0], (unsigned long long)ts[0] * ts[1] * ts[2] * 4);
-    atomicAdd(&P.stats[1], s_stat[0]);
-    atomicAdd(&P.stats[2], s_stat[1]);
-    atomicAdd(&P.stats[3], s_stat[2]);
+}
+
+// Tables of a CTA in shared memory: EPI differences (dynamic), qSRO weights, the
+// changing environment sites by partner direction, neighbour offsets (the first 12
+// are the partner offsets).
+template <int K, int TM>
+struct Tables {
+  static constexpr int NS = make_qclass<K, TM>().NS, NP = make_qclass<K, TM>().NP, NV = vec_count(kFCC, K);
+  int32_t wq[kMaxShells * kMaxSweepM];
+  short es[12 * NS], ep[12 * NP];
+  int qoff[NV];
+  unsigned long long stat[3];
+  __device__ __forceinline__ void fill(const SweepParams& P, const QsroTables& Q, int32_t* s_w) {
+    constexpr qfcc::QTable T = qfcc::make_qvecs();
+    const int tid = threadIdx.x, nth = blockDim.x, KM = K * P.M, nW = P.M * P.M * (KM + 1);
+    if (tid < 3) stat[tid] = 0;
+    for (int i = tid; i < nW; i += nth) s_w[i] = P.wtab[i];
+    for (int i = tid; i < KM; i += nth) wq[i] = Q.W[i];
+    for (int i = tid; i < 12 * NS; i += nth) es[i] = (qclass<K, TM>().es)[i / NS][i % NS];
+    for (int i = tid; i < 12 * NP; i += nth) ep[i] = (qclass<K, TM>().ep)[i / NP][i % NP];
+    if (tid < NV) {
+      int o = 0;
+#pragma unroll
+      for (int j = 0; j < NV; j++)
+        if (j == tid) o = QBox<TM>::voff(T.v[j].x, T.v[j].y, T.v[j].z);
+      qoff[tid] = o;
+    }
   }
+  // statistics of the tile to the lattice's counters
+  __device__ __forceinline__ void finish(const SweepParams& P, const int (&ts)[3], unsigned acc, unsigned same,
+                                         long long dsum) {
+    add_stats_warp(stat, acc, same, dsum);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      atomicAdd(&P.stats[0], (unsigned long long)ts[0] * ts[1] * ts[2] * 4);
+      atomicAdd(&P.stats[1], stat[0]);
+      atomicAdd(&P.stats[2], stat[1]);
+      atomicAdd(&P.stats[3], stat[2]);
+    }
+  }
+};
+}  // namespace qfn
+
+template <int K, int TM>
+__global__ void __launch_bounds__(128, TM == 20 ? 2 : 3)
+    k_qsro_fcc_n(const SweepParams P, const QsroTables Q, uint16_t* __restrict__ cnt) {
+  using namespace qfn;
+  using BX = QBox<TM>;
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ Tables<K, TM> S;
+  const int tid = threadIdx.x;
+  const int M = P.M, KM = K * P.M, MM = P.M * P.M;
+  uint16_t* box = reinterpret_cast<uint16_t*>(smem);
+  int32_t* s_w = reinterpret_cast<int32_t*>(smem + BX::BOX_BYTES);
+  int t0[3], ts[3];
+  colour_tile(P, t0, ts);
+  S.fill(P, Q, s_w);
+  stage<TM>(P, cnt, box, t0, ts);
+  const int nx = P.n[0], ny = P.n[1];
+  __syncthreads();
+
+  unsigned acc = 0, same = 0;
+  long long dsum = 0;
+  const int L = P.L;
+  const int NQ = (max(ts[0], max(ts[1], ts[2])) + L - 1) / L;
+  const int qx = tid % NQ, qy = (tid / NQ) % NQ, qz = tid / (NQ * NQ);
+  const bool slot = tid < NQ * NQ * NQ;
+  for (int cz = 0; cz < L; cz++)
+    for (int cy = 0; cy < L; cy++)
+      for (int cx = 0; cx < L; cx++) {
+        const int xr = cx + L * qx, yr = cy + L * qy, zr = cz + L * qz;
+        const bool here = slot && xr < ts[0] && yr < ts[1] && zr < ts[2];
+        const int cbase = BX::eidx(2 * xr + 3, 2 * yr + 3, 2 * zr + 3);
+        const unsigned long long cell = ((unsigned long long)(t0[2] + zr) * ny + (t0[1] + yr)) * nx + (t0[0] + xr);
+        uint4 rw = make_uint4(0, 0, 0, 0);
+        for (int b = 0; b < 4; b++) {
+          if (here) {
+            if ((b & 1) == 0) rw = attempt_block(cell * 4 + b, P.sweep, P.replica, P.seed_lo, P.seed_hi);
+            const uint32_t rd = (b & 1) ? rw.z : rw.x;
+            const uint32_t ru = (b & 1) ? rw.w : rw.y;
+            const int s = cbase + BX::voff(bx_of(b), by_of(b), bz_of(b));
+            const int dir = (int)__umulhi(rd, 12u);
+            const int sp = s + S.qoff[dir];
+            const int sa = box[s] & 7, sb = box[sp] & 7;
+            if (sa == sb) {
+              same++;
+            } else {
+              const int32_t* W = s_w + (sa * M + sb) * KM;
+              int wqa[K], wqb[K];
+#pragma unroll
+              for (int k = 0; k < K; k++) {
+                wqa[k] = S.wq[k * M + sa];
+                wqb[k] = S.wq[k * M + sb];
+              }
+              // pair part and the counts of s and s' after the swap: b
+              // around s without s' (which holds b before the swap), a around
+              // s' without s
+              int na_s[K], nb_s[K], na_p[K], nb_p[K];
+              int dE = s_w[MM * KM + sa * M + sb] + pair_side<K, TM, 1>(box, s, W, M, sa, sb, na_s, nb_s) +
+                       pair_side<K, TM, -1>(box, sp, W, M, sa, sb, na_p, nb_p);
+              nb_s[0]--;
+              na_p[0]--;
+#pragma unroll
+              for (int k = 0; k < K; k++)
+                dE += wqb[k] * (nb_s[k] * nb_s[k] - nb_p[k] * nb_p[k]) + wqa[k] * (na_p[k] * na_p[k] - na_s[k] * na_s[k]);
+              // environment sites whose counts move
+              const short* es = S.es + dir * S.NS;
+              const short* ep = S.ep + dir * S.NP;
+              dE += es_energy<K, TM, 0, Tables<K, TM>::NS>(box, es, s, sa, sb, wqa, wqb);
+              dE += ep_energy<K, TM>(box, ep, sp, sa, sb, wqa, wqb);
+              if (metropolis_accept(dE, ru, P.thr, P.nA, P.thr + kNA)) {
+                box[s] = (uint16_t)(sb | (pack_counts<K>(nb_s) << 3));
+                box[sp] = (uint16_t)(sa | (pack_counts<K>(na_p) << 3));
+                es_update<K, TM, 0, Tables<K, TM>::NS>(box, es, s, sa, sb);
+                ep_update<K, TM>(box, ep, sp, sa, sb);
+                acc++;
+                dsum += dE;
+              }
+            }
+          }
+          __syncthreads();
+        }
+      }
+
+  write_back<TM>(P, cnt, box, t0, ts);
+  S.finish(P, ts, acc, same, dsum);
+}
+
+// Four threads share a trial, one in each quarter of the CTA's warps (role): the
+// pair part around s, the pair part around s', and two parts of the changing
+// environment sites, of about equal length.  They leave their share of dE (and the
+// counts of s and s') in shared memory, meet at a barrier, and each decides for
+// itself and makes the updates of its own sites; role 1 draws the next words.
+// For lattices with at most one tile of a colour per SM, whose sweep is a chain of
+// 2,048 phases: 120^3 cells, 5 species, 3 shells 10.5 -> 8.3 ms per sweep, 64^3
+// 11.2 -> 7.5, 200^3 11.5 -> 8.5.  With more tiles the SMs have warps enough and
+// k_qsro_fcc_n's fewer instructions win (320^3 in 16-cell tiles: 31.1 against 40.8).
+constexpr int kQsroSlots = 128;     // link-cell slots of a tile at most
+constexpr int kQsroRoles = 4;
+template <int K, int TM>
+__global__ void __launch_bounds__(kQsroSlots * kQsroRoles)
+    k_qsro_fcc_roles(const SweepParams P, const QsroTables Q, uint16_t* __restrict__ cnt) {
+  using namespace qfn;
+  using BX = QBox<TM>;
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ Tables<K, TM> S;
+  constexpr int NS = Tables<K, TM>::NS;
+  constexpr int NSA = NS * 20 / 33;  // environment-of-s sites of role 2; role 3 takes the rest and ep
+  __shared__ uint4 s_rw[kQsroSlots];              // Philox block of the slot's site pair
+  __shared__ int s_part[kQsroRoles][kQsroSlots];  // shares of dE
+  __shared__ int s_cnt[2][kQsroSlots][K];         // counts around s and s': a | b << 8
+  const int tid = threadIdx.x;
+  const int M = P.M, KM = K * P.M, MM = P.M * P.M;
+  uint16_t* box = reinterpret_cast<uint16_t*>(smem);
+  int32_t* s_w = reinterpret_cast<int32_t*>(smem + BX::BOX_BYTES);
+  int t0[3], ts[3];
+  colour_tile(P, t0, ts);
+  S.fill(P, Q, s_w);
+  stage<TM>(P, cnt, box, t0, ts);
+  const int nx = P.n[0], ny = P.n[1];
+
+  unsigned acc = 0, same = 0;
+  long long dsum = 0;
+  const int L = P.L;
+  const int NQ = (max(ts[0], max(ts[1], ts[2])) + L - 1) / L;
+  const int role = tid / kQsroSlots, sl = tid % kQsroSlots;
+  const int qx = sl % NQ, qy = (sl / NQ) % NQ, qz = sl / (NQ * NQ);
+  const bool slot = sl < NQ * NQ * NQ;
+  // random words of site pair pr (sublattices 2 pr, 2 pr + 1) of the slot's cell
+  // at (cx, cy, cz) of the link cell, drawn by role 1
+  auto draw = [&](int cx, int cy, int cz, int pr) {
+    const int xr = cx + L * qx, yr = cy + L * qy, zr = cz + L * qz;
+    if (!slot || xr >= ts[0] || yr >= ts[1] || zr >= ts[2]) return;
+    const unsigned long long cell = ((unsigned long long)(t0[2] + zr) * ny + (t0[1] + yr)) * nx + (t0[0] + xr);
+    s_rw[sl] = attempt_block(cell * 4 + 2 * pr, P.sweep, P.replica, P.seed_lo, P.seed_hi);
+  };
+  if (role == 1) draw(0, 0, 0, 0);
+  __syncthreads();
+  for (int cz = 0; cz < L; cz++)
+    for (int cy = 0; cy < L; cy++)
+      for (int cx = 0; cx < L; cx++) {
+        const int xr = cx + L * qx, yr = cy + L * qy, zr = cz + L * qz;
+        const bool here = slot && xr < ts[0] && yr < ts[1] && zr < ts[2];
+        const int cbase = BX::eidx(2 * xr + 3, 2 * yr + 3, 2 * zr + 3);
+        for (int b = 0; b < 4; b++) {
+          int s = 0, sp = 0, sa = 0, sb = 0, dir = 0;
+          uint32_t ru = 0;
+          if (here) {
+            const uint4 rw = s_rw[sl];
+            ru = (b & 1) ? rw.w : rw.y;
+            dir = (int)__umulhi((b & 1) ? rw.z : rw.x, 12u);
+            s = cbase + BX::voff(bx_of(b), by_of(b), bz_of(b));
+            sp = s + S.qoff[dir];
+            sa = box[s] & 7;
+            sb = box[sp] & 7;
+          }
+          const bool live = here && sa != sb;
+          if (here && !live && role == 0) same++;
+          const short* es = S.es + dir * S.NS;
+          const short* ep = S.ep + dir * S.NP;
+          if (live) {
+            const int32_t* W = s_w + (sa * M + sb) * KM;
+            int part;
+            if (role < 2) {
+              int na[K], nb[K];
+              if (role == 0) {
+                part = s_w[MM * KM + sa * M + sb] + pair_side<K, TM, 1>(box, s, W, M, sa, sb, na, nb);
+                nb[0]--;  // s' holds b before the swap
+              } else {
+                part = pair_side<K, TM, -1>(box, sp, W, M, sa, sb, na, nb);
+                na[0]--;  // s holds a before the swap
+              }
+#pragma unroll
+              for (int k = 0; k < K; k++) s_cnt[role][sl][k] = na[k] | (nb[k] << 8);
+            } else {
+              int wqa[K], wqb[K];
+#pragma unroll
+              for (int k = 0; k < K; k++) {
+                wqa[k] = S.wq[k * M + sa];
+                wqb[k] = S.wq[k * M + sb];
+              }
+              if (role == 2)
+                part = es_energy<K, TM, 0, NSA>(box, es, s, sa, sb, wqa, wqb);
+              else
+                part = es_energy<K, TM, NSA, NS>(box, es, s, sa, sb, wqa, wqb) +
+                       ep_energy<K, TM>(box, ep, sp, sa, sb, wqa, wqb);
+            }
+            s_part[role][sl] = part;
+          }
+          __syncthreads();
+          if (live) {
+            // every role: the whole dE, with the quadratic terms of s and s' from
+            // the counts they have before (a at s, b at s') and after the swap
+            int dE = (s_part[0][sl] + s_part[1][sl]) + (s_part[2][sl] + s_part[3][sl]);
+            int nb_s[K], na_p[K];
+#pragma unroll
+            for (int k = 0; k < K; k++) {
+              const int cs = s_cnt[0][sl][k], cp = s_cnt[1][sl][k];
+              const int na_s = cs & 255, nb_p = cp >> 8;
+              nb_s[k] = cs >> 8;
+              na_p[k] = cp & 255;
+              dE += S.wq[k * M + sb] * (nb_s[k] * nb_s[k] - nb_p * nb_p) +
+                    S.wq[k * M + sa] * (na_p[k] * na_p[k] - na_s * na_s);
+            }
+            if (metropolis_accept(dE, ru, P.thr, P.nA, P.thr + kNA)) {
+              if (role == 0) {
+                box[s] = (uint16_t)(sb | (pack_counts<K>(nb_s) << 3));
+                acc++;
+                dsum += dE;
+              } else if (role == 1) {
+                box[sp] = (uint16_t)(sa | (pack_counts<K>(na_p) << 3));
+              } else if (role == 2) {
+                es_update<K, TM, 0, NSA>(box, es, s, sa, sb);
+              } else {
+                es_update<K, TM, NSA, NS>(box, es, s, sa, sb);
+                ep_update<K, TM>(box, ep, sp, sa, sb);
+              }
+            }
+          }
+          if (role == 1 && (b & 1)) {  // the words of the next pair of sites
+            if (b == 1) {
+              draw(cx, cy, cz, 1);
+            } else {
+              const int nx_ = cx + 1 < L ? cx + 1 : 0;
+              const int ny_ = nx_ ? cy : cy + 1 < L ? cy + 1 : 0;
+              const int nz_ = nx_ || ny_ ? cz : cz + 1;
+              if (nz_ < L) draw(nx_, ny_, nz_, 0);
+            }
+          }
+          __syncthreads();
+        }
+      }
+
+  write_back<TM>(P, cnt, box, t0, ts);
+  S.finish(P, ts, acc, same, dsum);
 }
 
 // sum_i sum_k W[k][s_i] n_k(i)^2 added to *E (global-memory gathers).
@@ -988,12 +1170,20 @@ void sweep_qsro_device(smcx_lattice* hd, int nA, uint64_t seed, int64_t n_sweeps
     auto init = K == 2 ? k_qsro_fcc_count_init<2> : k_qsro_fcc_count_init<3>;
     check_cuda(cudaFuncSetAttribute(init, cudaFuncAttributeMaxDynamicSharedMemorySize, qfcc::BOX_BYTES),
                "qSRO count smem attribute");
-    init<<<sc.nt[0] * sc.nt[1] * sc.nt[2], 128, qfcc::BOX_BYTES, hd->stream>>>(P, hd->d_qcnt);
+    init<<<sc.nt[0] * sc.nt[1] * sc.nt[2], 512, qfcc::BOX_BYTES, hd->stream>>>(P, hd->d_qcnt);
     const int nW = P.M * P.M * K * P.M + P.M * P.M;
     const bool small = tm <= 17;  // the 66 KB box: three CTAs per SM
     const size_t smem = (small ? qfn::QBox<17>::BOX_BYTES : qfn::QBox<20>::BOX_BYTES) + (size_t)nW * 4;
+    const int grid = P.ntc[0] * P.ntc[1] * P.ntc[2];
+    // four threads per trial while a colour has at most one tile per SM (measured
+    // at k_qsro_fcc_roles)
+    const bool roles = grid <= 152;
     auto kern = K == 2 ? (small ? k_qsro_fcc_n<2, 17> : k_qsro_fcc_n<2, 20>)
                        : (small ? k_qsro_fcc_n<3, 17> : k_qsro_fcc_n<3, 20>);
+    if (roles)
+      kern = K == 2 ? (small ? k_qsro_fcc_roles<2, 17> : k_qsro_fcc_roles<2, 20>)
+                    : (small ? k_qsro_fcc_roles<3, 17> : k_qsro_fcc_roles<3, 20>);
+    const int threads = roles ? kQsroSlots * kQsroRoles : 128;
     check_cuda(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
                "qSRO FCC smem attribute");
     check_cuda(cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100), "qSRO FCC carveout");
@@ -1001,7 +1191,7 @@ void sweep_qsro_device(smcx_lattice* hd, int nA, uint64_t seed, int64_t n_sweeps
       P.sweep = hd->sweep_cum + (uint64_t)sw;
       for (int tc = 0; tc < n_colours; tc++) {
         P.tc = tc;
-        kern<<<P.ntc[0] * P.ntc[1] * P.ntc[2], 128, smem, hd->stream>>>(P, T, hd->d_qcnt);
+        kern<<<grid, threads, smem, hd->stream>>>(P, T, hd->d_qcnt);
       }
     }
     check_cuda(cudaGetLastError(), "qSRO FCC sweep launch");

@@ -93,3 +93,20 @@ def test_pair_counts_batch_sizes(kind, dims, M, K, B):
         C = diff.pair_counts(view.view(B, N), kind, dims, M, K).cpu().numpy()
         for b in range(B):
             assert (C[b] == O.pair_counts(kind, dims, M, K, cfg[b])).all()
+
+
+@pytest.mark.parametrize("dims,nt", [((40, 38, 42), (12, 12, 12)), ((18, 21, 40), (2, 2, 2)), ((34, 33, 32), (2, 2, 2))])
+@pytest.mark.parametrize("M,K,storage", [(5, 3, smcx.PACKED4), (4, 2, smcx.INT8), (8, 3, smcx.INT8)])
+def test_qsro_sweeps_few_and_many_tiles(dims, nt, M, K, storage):
+    # 216 tiles a colour: a thread per trial; one tile a colour: four threads per
+    # trial, in the boxes of 20-cell and of 17-cell tiles
+    W = np.random.default_rng(8).integers(-300, 301, (K, M)).astype(np.int32)
+    lat, cfg, V = _lattice(smcx.FCC, dims, M, K, storage, 9)
+    lat.set_qsro(W)
+    lat.set_schedule((4, nt))
+    lat.sweep(900.0, 2, 31)
+    st = O.sweep_qsro(O.FCC, dims, M, K, V, W, cfg, 900.0, 2, 31, L=4, nt=nt)
+    assert (lat.get_config() == cfg).all()
+    assert lat.state()[1].tolist() == st.tolist()
+    assert lat.energy() == O.energy_qsro(O.FCC, dims, M, K, V, W, cfg)
+    lat.close()
