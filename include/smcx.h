@@ -402,7 +402,8 @@ int smcx_threshold_tables(double T, uint32_t* A, int* nA, uint32_t* B);
  *                       slot per thread).
  *   smcx_batch_sweep    n_sweeps at temperatures T[R] with Philox seed `seed`;
  *                       returns after the launch has finished; SMCX_E_TIMEOUT
- *                       if a grid barrier waited longer than its limit.
+ *                       if a tile pass waited longer than the limit for
+ *                       the tiles of its replica that come before it.
  *   smcx_batch_autotune times `trial_sweeps` batched sweeps for every
  *                       candidate (link cell 3 or 4, tiles of at most 12-20
  *                       cells, 128- or 256-thread CTAs) on snapshots of the

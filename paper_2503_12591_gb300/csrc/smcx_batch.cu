@@ -8,12 +8,11 @@
 // sweep counter and Philox replica id, so its trajectory is bit-identical to
 // sweeping it alone through smcx_sweep, in either proposal mode.
 //
-// The kernel (smcx_batch_body.cuh) loops over sweeps and tile colours; in
-// each colour the CTAs take the pooled list of (replica, tile) work items of
-// that colour, then meet at a grid barrier.  The barrier waits at most
-// `timeout_ns`: a CTA that gives up writes SMCX_E_TIMEOUT into a device status
-// word and returns, and so does every other CTA once it sees the status, so
-// the context stays usable.
+// The kernel (smcx_batch_body.cuh) works through one list of tile passes, the
+// pooled (replica, tile) items of every sweep and colour; a pass waits for its own
+// replica's previous colour only.  A wait lasts at most `timeout_ns`: a CTA that
+// gives up writes SMCX_E_TIMEOUT into a device status word and returns, and so does
+// every other CTA once it sees the status, so the context stays usable.
 #include <algorithm>
 #include <cmath>
 #include <map>
@@ -26,11 +25,11 @@ struct smcx_batch {
   smcx::bccfast::LatDesc* d_desc = nullptr;
   int2* d_items = nullptr;  // (replica, tile index within its colour)
   int n_items = 0;
-  unsigned* d_bar = nullptr;
+  smcx::bccfast::Progress* d_progress = nullptr;
   int* d_status = nullptr;
   int threads = 0, slots = 1;
   long long timeout_ns = 2000000000ll;
-  int skip_cta = -1;  // fault injection: this CTA never arrives at the barrier
+  int skip_cta = -1;  // fault injection: this CTA never reports its tile pass as done
   bool use_graph = true;
   std::map<long long, cudaGraphExec_t> graphs;  // keyed by (sweeps, table size)
   std::vector<int32_t> graph_V;                 // EPI baked into the graphs
@@ -146,7 +145,7 @@ static void batch_sweep_launch(smcx_batch* b, const double* T, int64_t n_sweeps,
 
 void batch_sweep(smcx_batch* b, const double* T, int64_t n_sweeps, uint64_t seed) {
   check_batch(b);
-  // at most 2^16 sweeps per launch keep the barrier counter far from overflow
+  // at most 2^16 sweeps per launch: the kernel counts colours in 32 bits
   for (int64_t done = 0; done < n_sweeps;) {
     const int64_t n = std::min<int64_t>(n_sweeps - done, 1 << 16);
     batch_sweep_launch(b, T, n, seed);
@@ -203,14 +202,14 @@ static void batch_sweep_launch(smcx_batch* b, const double* T, int64_t n_sweeps,
   check_cuda(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void*)fn, b->threads, smem), "occupancy");
   if (per_sm < 1) fail(SMCX_E_UNSUPPORTED, "batch kernel does not fit an SM");
   const int grid = std::min(b->n_items, per_sm * nsm);
-  if (!b->d_bar) {
-    check_cuda(cudaMalloc(&b->d_bar, sizeof(unsigned)), "barrier word");
+  if (!b->d_progress) {
+    check_cuda(cudaMalloc(&b->d_progress, bccfast::progress_bytes(R)), "batch progress counters");
     check_cuda(cudaMalloc(&b->d_status, sizeof(int)), "status word");
   }
   int n_int = (int)n_sweeps;
   int max_nA_arg = nA_cap;
   void* args[] = {(void*)&Q, (void*)&b->d_desc, (void*)&b->d_items, (void*)&b->n_items, (void*)&n_int,
-                  (void*)&b->d_bar, (void*)&b->d_status, (void*)&b->timeout_ns, (void*)&b->skip_cta,
+                  (void*)&b->d_progress, (void*)&b->d_status, (void*)&b->timeout_ns, (void*)&b->skip_cta,
                   (void*)&max_nA_arg};
   if (b->graph_V != b->lat[0]->V) {
     for (auto& g : b->graphs) cudaGraphExecDestroy(g.second);
@@ -218,7 +217,7 @@ static void batch_sweep_launch(smcx_batch* b, const double* T, int64_t n_sweeps,
     b->graph_V = b->lat[0]->V;
   }
   auto enqueue = [&]() {
-    check_cuda(cudaMemsetAsync(b->d_bar, 0, sizeof(unsigned), b->stream), "barrier reset");
+    check_cuda(cudaMemsetAsync(b->d_progress, 0, bccfast::progress_bytes(R), b->stream), "progress reset");
     check_cuda(cudaMemsetAsync(b->d_status, 0, sizeof(int), b->stream), "status reset");
     check_cuda(cudaLaunchCooperativeKernel((const void*)fn, dim3(grid), dim3(b->threads), args, smem, b->stream),
                "batch cooperative launch");
@@ -235,7 +234,7 @@ static void batch_sweep_launch(smcx_batch* b, const double* T, int64_t n_sweeps,
       cudaGraphExec_t ge = nullptr;
       bool ok = cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
       if (ok) {
-        cudaMemsetAsync(b->d_bar, 0, sizeof(unsigned), b->stream);
+        cudaMemsetAsync(b->d_progress, 0, bccfast::progress_bytes(R), b->stream);
         cudaMemsetAsync(b->d_status, 0, sizeof(int), b->stream);
         cudaLaunchCooperativeKernel((const void*)fn, dim3(grid), dim3(b->threads), args, smem, b->stream);
         ok = cudaStreamEndCapture(b->stream, &g) == cudaSuccess && g != nullptr;
@@ -257,7 +256,7 @@ static void batch_sweep_launch(smcx_batch* b, const double* T, int64_t n_sweeps,
   int status = 0;
   check_cuda(cudaMemcpyAsync(&status, b->d_status, sizeof(int), cudaMemcpyDeviceToHost, b->stream), "status read");
   check_cuda(cudaStreamSynchronize(b->stream), "batch sync");
-  if (status != 0) fail(status, "batched sweep stopped: a grid barrier timed out");
+  if (status != 0) fail(status, "batched sweep stopped: a tile pass waited too long for its replica");
   for (smcx_lattice* h : b->lat) h->sweep_cum += (uint64_t)n_sweeps;
 }
 
@@ -268,7 +267,7 @@ void batch_release(smcx_batch* b) {
   cudaFree(b->d_fdesc);
   cudaFree(b->d_fitems);
   cudaFree(b->d_fcounts);
-  cudaFree(b->d_bar);
+  cudaFree(b->d_progress);
   cudaFree(b->d_status);
 }
 

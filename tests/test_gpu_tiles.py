@@ -110,3 +110,35 @@ def test_qsro_sweeps_few_and_many_tiles(dims, nt, M, K, storage):
     assert lat.state()[1].tolist() == st.tolist()
     assert lat.energy() == O.energy_qsro(O.FCC, dims, M, K, V, W, cfg)
     lat.close()
+
+
+@pytest.mark.parametrize("proposal,R,lo,hi,tile", [(0, 40, 24, 66, 12), (1, 40, 24, 66, 12), (2, 33, 12, 72, 14), (1, 1, 16, 16, 8),
+                                                   (0, 600, 12, 12, 6)])
+def test_batch_list_longer_than_the_grid(proposal, R, lo, hi, tile):
+    # tile passes drawn from the list by CTAs that run ahead of other replicas
+    stream = torch.cuda.current_stream()
+    V = epi_gaussian(4, 4, 20.0, 2)
+    edges = np.linspace(lo, hi, R).astype(int)
+
+    def lattice(r):
+        n = int(edges[r])
+        nt = 2 * -(-n // (2 * tile))
+        lat = smcx.Lattice(smcx.BCC, (n, n, n), 4, [0.25] * 4, init_seed=50 + r, storage=smcx.PACKED4,
+                           sched=(3, (nt, nt, nt)), stream=stream)
+        lat.set_replica(r)
+        lat.set_epi(V)
+        lat.set_proposal(proposal)
+        return lat
+
+    T = np.linspace(400.0, 2400.0, R)
+    lats = [lattice(r) for r in range(R)]
+    b = smcx.Batch(lats, stream)
+    b.sweep(T, 1, 9)
+    b.sweep(T, 3, 9)
+    for r in range(0, R, max(1, R // 20)):
+        one = lattice(r)
+        one.sweep(T[r], 4, 9)
+        assert (lats[r].get_config() == one.get_config()).all()
+        assert lats[r].state()[1].tolist() == one.state()[1].tolist()
+        one.close()
+    b.close()
