@@ -35,40 +35,82 @@ constexpr int PZ = 24;             // planes
 constexpr int SUB = PP * PZ;       // bytes per sublattice array
 constexpr int BOX = 24;            // usable box edge (tile <= 20 with halo 2)
 
-// Lane order of the 5^3 link-cell slots of a 20-cell tile (L = 4) on a
-// 128-thread CTA: slot kSlotOrder[t] for thread t (255: none).  Slot q =
-// (qx, qy, qz) = (q % 5, q / 5 % 5, q / 25) starts at byte qx 4 + qy 4 PX +
-// qz 4 PP of the box, i.e. word qx + qy PX + qz PP; the order gives the 32
-// lanes of every warp 32 different banks, so a neighbour load at a common
-// offset (all loads of the centre environment) is one wavefront.  Any order
-// gives the same result: the trials of a phase are independent.
-#define SMCX_BCC_SLOT_ORDER                                                                                          \
-  0, 1, 2, 3, 4, 21, 22, 23, 24, 29, 46, 15, 16, 17, 18, 19, 40, 41, 10, 11, 12, 13, 14, 35, 36, 5, 6, 7, 8, 9, 30, 31, 32, 33, 34, 55, 20, 25, 26, 27, 28, 45, 50, 47, 48, 49, 54, 71, 72, 73, 42, 43, 44, 65, 66, 67, 68, 37, 38, 39, 60, 61, 62, 63, 64, 85, 86, 87, 56, 57, 58, 59, 80, 81, 82, 51, 52, 53, 70, 75, 76, 77, 74, 79, 96, 97, 98, 99, 104, 69, 90, 91, 92, 93, 94, 115, 116, 117, 118, 119, 88, 89, 110, 111, 112, 113, 114, 83, 84, 105, 106, 107, 108, 109, 78, 95, 100, 101, 102, 103, 120, 121, 122, 123, 124, 255, 255, 255
-constexpr unsigned char kSlotOrder[128] = {SMCX_BCC_SLOT_ORDER};
-static __constant__ unsigned char c_slot_order[128] = {SMCX_BCC_SLOT_ORDER};
-__host__ __device__ constexpr bool slot_order_ok() {
-  for (int w = 0; w < 4; w++) {
-    bool seen[32] = {};
-    for (int l = 0; l < 32; l++) {
-      const int q = kSlotOrder[32 * w + l];
-      if (q == 255) continue;
-      const int bank = (q % 5 + PX * (q / 5 % 5) + PP * (q / 25)) % 32;
-      if (seen[bank]) return false;
-      seen[bank] = true;
+// Lane orders of the NQ^3 link-cell slots of a tile: entry t is the slot of thread t
+// (255: none).  Slot q = (qx, qy, qz) = (q % NQ, q / NQ % NQ, q / NQ^2) starts at byte
+// L (qx + qy PX + qz PP) of the box, and all loads of a centre's environment are at
+// that place plus an offset common to the warp.  One pass over the slots fills warp
+// after warp with lanes whose words lie in different banks (or in the same word) for
+// all four byte offsets within a word; lanes that would clash stay idle while the
+// remaining warps have room, then `clash` lanes may share a bank.  Any order gives the
+// same result: the trials of a phase are independent.
+// Shared loads bound a sweep that fills the GPU.  A load at a common offset takes 2.0
+// wavefronts in plain order for a full tile of 4^3 or 5^3 slots and 1.7 for 6^3; in
+// these orders 1.0 (5^3, L = 4), 1.14 (6^3, L = 3), 1.25 (5^3, L = 3), 1.5 (4^3, L = 4).
+// Sweeps of 400^3 cells, plain and ordered: 15-cell tiles L = 3 4.01 and 3.68 ms (shared
+// directions 2.69 and 2.33), 18-cell tiles L = 3 4.25 and 3.83 ms; 256^3 cells, 16-cell
+// tiles L = 4 1.37 and 1.21 ms.  Shapes outside the table gained less or nothing.
+constexpr int kOrderMinNQ = 4, kOrderMaxNQ = 6, kOrderMinL = 3, kOrderMaxL = 5;
+__host__ __device__ constexpr int order_lanes(int nq) { return (nq * nq * nq + 31) / 32 * 32; }
+
+struct SlotOrders {
+  unsigned char q[kOrderMaxNQ - kOrderMinNQ + 1][kOrderMaxL - kOrderMinL + 1][224];
+};
+__host__ __device__ constexpr SlotOrders make_slot_orders() {
+  SlotOrders T{};
+  for (int nq = kOrderMinNQ; nq <= kOrderMaxNQ; nq++)
+    for (int L = kOrderMinL; L <= kOrderMaxL; L++) {
+      unsigned char* out = T.q[nq - kOrderMinNQ][L - kOrderMinL];
+      for (int t = 0; t < 224; t++) out[t] = 255;
+      const int n = nq * nq * nq, warps = order_lanes(nq) / 32;
+      bool used[216] = {};
+      int left = n;
+      for (int w = 0; w < warps; w++) {
+        int word[4][32][8] = {}, words[4][32] = {};  // distinct words per bank, per byte offset
+        int lanes = 0;
+        for (int clash = 1; lanes < 32 && left > 0; clash++) {
+          for (int q = 0; q < n && lanes < 32; q++) {
+            if (used[q]) continue;
+            bool fits = true, is_new[4] = {};
+            int at[4] = {};
+            for (int o = 0; o < 4; o++) {
+              at[o] = (L * (q % nq + q / nq % nq * PX + q / (nq * nq) * PP) + o) / 4;
+              is_new[o] = true;
+              for (int i = 0; i < words[o][at[o] % 32]; i++)
+                if (word[o][at[o] % 32][i] == at[o]) is_new[o] = false;
+              if (is_new[o] && words[o][at[o] % 32] >= clash) fits = false;
+            }
+            if (!fits) continue;
+            for (int o = 0; o < 4; o++)
+              if (is_new[o]) word[o][at[o] % 32][words[o][at[o] % 32]++] = at[o];
+            used[q] = true;
+            out[32 * w + lanes++] = (unsigned char)q;
+            left--;
+          }
+          if (left <= 32 * (warps - 1 - w)) break;  // the rest fits into the other warps
+        }
+      }
     }
-  }
-  bool used[125] = {};
-  for (int t = 0; t < 128; t++) {
-    const int q = kSlotOrder[t];
-    if (q == 255) continue;
-    if (q >= 125 || used[q]) return false;
-    used[q] = true;
-  }
-  for (int q = 0; q < 125; q++)
-    if (!used[q]) return false;
+  return T;
+}
+constexpr SlotOrders kSlotOrders = make_slot_orders();
+static __device__ const SlotOrders d_slot_orders = kSlotOrders;
+__host__ __device__ constexpr bool slot_orders_ok() {
+  for (int nq = kOrderMinNQ; nq <= kOrderMaxNQ; nq++)
+    for (int L = kOrderMinL; L <= kOrderMaxL; L++) {
+      bool used[256] = {};
+      int n = 0;
+      for (int t = 0; t < order_lanes(nq); t++) {
+        const int q = kSlotOrders.q[nq - kOrderMinNQ][L - kOrderMinL][t];
+        if (q == 255) continue;
+        if (q >= nq * nq * nq || used[q]) return false;
+        used[q] = true;
+        n++;
+      }
+      if (n != nq * nq * nq) return false;
+    }
   return true;
 }
-static_assert(slot_order_ok(), "slot order must cover the 125 slots with distinct banks per warp");
+static_assert(slot_orders_ok(), "a lane order must hold every slot once");
 constexpr int MAXPLANES = 3;
 
 // Byte planes of the EPI table, shared by every lattice of a launch:
@@ -518,6 +560,22 @@ __device__ __forceinline__ void bcc_tile_pass(const LatDesc& D, const Planes& Q,
     ts[a] = base + (ti[a] < rem ? 1 : 0);
     t0[a] = ti[a] * base + min(ti[a], rem);
   }
+  // link-cell slots of this thread, in the bank-spreading order where the shape has
+  // one.  Shared-direction passes read it before the tile is staged, which hides the
+  // load; passes with a direction per trial have no registers to hold it.
+  const int NQ = D.NQ, L = D.L;
+  const bool ordered = NQ >= kOrderMinNQ && NQ <= kOrderMaxNQ && L >= kOrderMinL && L <= kOrderMaxL &&
+                       nth * SLOTS >= order_lanes(NQ);
+  auto slot_of = [&](int j) {
+    const int t = tid + j * nth;
+    if (!ordered) return t;
+    return t < order_lanes(NQ) ? (int)d_slot_orders.q[NQ - kOrderMinNQ][L - kOrderMinL][t] : 255;
+  };
+  int q_early[PROP == 1 ? SLOTS : 1];
+  if (PROP == 1) {
+#pragma unroll
+    for (int j = 0; j < SLOTS; j++) q_early[j] = slot_of(j);
+  }
   __syncthreads();  // the previous pass of this CTA is done with the tables
   if (tid < 3) s_stat[tid] = 0;
   if (TL1) {
@@ -549,16 +607,11 @@ __device__ __forceinline__ void bcc_tile_pass(const LatDesc& D, const Planes& Q,
   stage_box(D, box, t0, ts, lane, warp, nwarp);
   __syncthreads();
 
-  // link-cell slots of this thread: q = tid + j * nth
-  const int NQ = D.NQ, L = D.L;
   int qx[SLOTS], qy[SLOTS], qz[SLOTS];
   bool slot[SLOTS];
-  // the bank-spreading lane order for the default shape (5^3 slots, 128
-  // threads, one slot each); plain order otherwise
-  const bool ordered = SLOTS == 1 && NQ == 5 && nth == 128;
 #pragma unroll
   for (int j = 0; j < SLOTS; j++) {
-    const int q = ordered ? (int)c_slot_order[tid] : tid + j * nth;
+    const int q = PROP == 1 ? q_early[PROP == 1 ? j : 0] : slot_of(j);
     qx[j] = q % NQ;
     qy[j] = (q / NQ) % NQ;
     qz[j] = q / (NQ * NQ);

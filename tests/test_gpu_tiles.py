@@ -142,3 +142,18 @@ def test_batch_list_longer_than_the_grid(proposal, R, lo, hi, tile):
         assert lats[r].state()[1].tolist() == one.state()[1].tolist()
         one.close()
     b.close()
+
+
+@pytest.mark.parametrize("L,nt,dims", [(3, 2, (24, 23, 22)), (3, 2, (30, 27, 25)), (3, 2, (36, 33, 31)), (4, 2, (32, 27, 29)),
+                                       (4, 2, (40, 33, 36)), (4, 4, (44, 43, 42)), (5, 2, (40, 34, 31)), (6, 2, (40, 38, 36))])
+@pytest.mark.parametrize("M,proposal,storage", [(4, 0, smcx.PACKED4), (4, 1, smcx.PACKED4), (4, 2, smcx.INT8), (6, 0, smcx.INT8)])
+def test_bcc_lane_orders(L, nt, dims, M, proposal, storage):
+    # 4^3 to 6^3 link-cell slots, full and ragged tiles; L = 6 has no order of its own
+    lat, cfg, V = _lattice(smcx.BCC, dims, M, 4, storage, 17)
+    lat.set_schedule((L, (nt, nt, nt)))
+    lat.set_proposal(proposal)
+    lat.sweep(1100.0, 2, 23)
+    st = O.sweep(O.BCC, dims, M, 4, V, cfg, 1100.0, 2, 23, L=L, nt=(nt, nt, nt), proposal=proposal)
+    assert (lat.get_config() == cfg).all()
+    assert lat.state()[1].tolist() == st.tolist()
+    lat.close()
