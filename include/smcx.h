@@ -421,11 +421,11 @@ int smcx_threshold_tables(double T, uint32_t* A, int* nA, uint32_t* B);
  *                       (one slot per thread; SMCX_E_UNSUPPORTED at the next
  *                       sweep if a tile has more than 256 link cells).
  *                       SMCX_E_INVALID_ARG for other values.
- *   smcx_batch_set_fault test hook: CTA `skip_cta` (>= 0) skips the first grid
- *                       barrier, which then times out after timeout_ms and the
- *                       next smcx_batch_sweep returns SMCX_E_TIMEOUT; -1 turns
- *                       it off.  timeout_ms (1..60000, default 2000) bounds
- *                       every barrier wait.
+ *   smcx_batch_set_fault test hook: CTA `skip_cta` (>= 0) never reports its first
+ *                       tile pass as done, so the wait of the passes that depend
+ *                       on it ends after timeout_ms and the next
+ *                       smcx_batch_sweep returns SMCX_E_TIMEOUT; -1 turns it off.
+ *                       timeout_ms (1..60000, default 2000) bounds every wait.
  */
 typedef struct smcx_batch smcx_batch;
 int smcx_batch_create(smcx_batch** out, int R, smcx_lattice* const* lattices, void* stream);

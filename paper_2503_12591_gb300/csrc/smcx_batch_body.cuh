@@ -5,7 +5,7 @@
 // trial body and constant-memory offset table live in that translation unit).
 #pragma once
 
-#include "smcx_bcc_tile.cuh"
+#include "smcx_bcc_group.cuh"
 
 namespace smcx {
 namespace bccfast {
@@ -118,6 +118,20 @@ __global__ void __launch_bounds__(256, 3)
   batch_body<K, NW, PL, 1, PROP>(Q, descs, items, n_items, n_sweeps, pr, status, timeout_ns, skip_cta, max_nA);
 }
 
+// Several lanes per trial (smcx_bcc_group.cuh), for few tiles of at most 3^3 slots.
+template <int LN, int K, int NW, int PL>
+__global__ void __launch_bounds__(kGroupThreads, 4)
+    k_bcc_batch_group(const Planes Q, const LatDesc* __restrict__ descs, const int2* __restrict__ items, int n_items,
+                      int n_sweeps, Progress* pr, int* status, long long timeout_ns, int skip_cta, int max_nA) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ __align__(16) GroupMem M;
+  uint32_t* sA = reinterpret_cast<uint32_t*>(smem + 2 * SUB);
+  batch_loop(descs, items, n_items, n_sweeps, pr, status, timeout_ns, skip_cta,
+             [&](const LatDesc& D, int tc, int jt, unsigned long long sweep) {
+               group_pass<LN, K, NW, PL>(D, Q, tc, jt, sweep, smem, sA, sA + max_nA, M);
+             });
+}
+
 using BatchKernelFn = void (*)(const Planes, const LatDesc*, const int2*, int, int, Progress*, int*, long long, int,
                                int);
 
@@ -126,5 +140,7 @@ using BatchKernelFn = void (*)(const Planes, const LatDesc*, const int2*, int, i
 // The shared-direction batch kernel (4 shells, M <= 4, two byte planes, one
 // link-cell slot per thread) for 128- or 256-thread CTAs.
 bccfast::BatchKernelFn batch_dir_kernel(int threads);  // smcx_sweep_bcc_dir.cu
+// Four lanes per trial (4 shells; nw counter words, pl byte planes).
+bccfast::BatchKernelFn batch_group_kernel(int nw, int pl);  // smcx_sweep_bcc_group.cu
 
 }  // namespace smcx

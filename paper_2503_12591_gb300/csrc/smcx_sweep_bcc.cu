@@ -1,6 +1,6 @@
 // Single-lattice BCC sweep on the specialised tile pass (smcx_bcc_tile.cuh):
 // one launch per tile colour, one CTA per tile of that colour.
-#include "smcx_bcc_tile.cuh"
+#include "smcx_bcc_group.cuh"
 
 namespace smcx {
 
@@ -95,6 +95,9 @@ void bcc_block_shape(int nq, int tuned_threads, int* threads, int* slots) {
 void sweep_bcc_dir(smcx_lattice* hd, bccfast::LatDesc& D, const bccfast::Planes& Q, int threads, int64_t n,
                    int nc);  // smcx_sweep_bcc_dir.cu
 
+void sweep_bcc_group(smcx_lattice* hd, bccfast::LatDesc& D, const bccfast::Planes& Q, int nw, int pl, int64_t n,
+                     int nc);  // smcx_sweep_bcc_group.cu
+
 static void dispatch(smcx_lattice* hd, bccfast::LatDesc& D, const bccfast::Planes& Q, int nw, int pl,
                      int threads, int slots, int64_t n, int nc) {
   const int K = hd->shells.K;
@@ -155,6 +158,14 @@ void sweep_bcc_fast(smcx_lattice* hd, int nA, uint64_t seed, int64_t n_sweeps, i
     nw = 2;
     PL = build_planes(hd, &Q, 3);
   }
+  // Several lanes per trial while the colour's tiles leave the GPU mostly idle: 3^3 slots
+  // up to two tiles per SM (216 tiles 0.443 -> 0.362 ms, 343 tiles 0.894 -> 0.907), 4^3
+  // slots up to one (125 tiles, L = 3 0.443 -> 0.394 ms, 216 tiles 0.469 -> 0.504).  A
+  // block size that was set is kept.
+  const int tiles = (sc.nt[0] / 2) * (sc.nt[1] / 2) * (sc.nt[2] / 2);
+  if (hd->bcc_threads == 0 && D.NQ <= bccfast::kMaxGroupNQ && tiles <= (D.NQ <= 3 ? 2 : 1) * kSMs &&
+      (D.proposal == 0 || D.L <= 6))
+    return sweep_bcc_group(hd, D, Q, nw, PL, n_sweeps, n_colours);
   int threads, slots;
   bcc_block_shape(D.NQ, hd->bcc_threads, &threads, &slots);
 

@@ -1177,7 +1177,7 @@ void sweep_qsro_device(smcx_lattice* hd, int nA, uint64_t seed, int64_t n_sweeps
     const int grid = P.ntc[0] * P.ntc[1] * P.ntc[2];
     // four threads per trial while a colour has at most one tile per SM (measured
     // at k_qsro_fcc_roles)
-    const bool roles = grid <= 152;
+    const bool roles = grid <= kSMs;
     auto kern = K == 2 ? (small ? k_qsro_fcc_n<2, 17> : k_qsro_fcc_n<2, 20>)
                        : (small ? k_qsro_fcc_n<3, 17> : k_qsro_fcc_n<3, 20>);
     if (roles)

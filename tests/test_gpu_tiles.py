@@ -157,3 +157,48 @@ def test_bcc_lane_orders(L, nt, dims, M, proposal, storage):
     assert (lat.get_config() == cfg).all()
     assert lat.state()[1].tolist() == st.tolist()
     lat.close()
+
+
+@pytest.mark.parametrize("L,nt,dims", [(3, 2, (6, 7, 9)), (4, 2, (12, 17, 24)), (6, 2, (36, 25, 31)), (3, 4, (24, 36, 33)),
+                                       (3, 2, (24, 23, 19)), (4, 2, (32, 29, 26)), (5, 2, (40, 31, 33)), (7, 2, (40, 39, 37)),
+                                       (3, 14, (84, 85, 86))])
+@pytest.mark.parametrize("M,K,proposal,storage", [(4, 4, 0, smcx.PACKED4), (4, 4, 1, smcx.INT8), (4, 3, 0, smcx.INT8),
+                                                  (6, 4, 0, smcx.PACKED4), (3, 2, 0, smcx.PACKED4), (5, 1, 0, smcx.INT8)])
+def test_bcc_lanes_per_trial(L, nt, dims, M, K, proposal, storage):
+    # two and four lanes per trial, and (84 cells in 14 tiles) one: 2^3 to 4^3 slots.
+    # Shared directions are held for link cells up to 6.
+    if proposal and L > 6:
+        return
+    lat, cfg, V = _lattice(smcx.BCC, dims, M, K, storage, 21)
+    lat.set_schedule((L, (nt, nt, nt)))
+    lat.set_proposal(proposal)
+    lat.sweep(1300.0, 2, 29)
+    st = O.sweep(O.BCC, dims, M, K, V, cfg, 1300.0, 2, 29, L=L, nt=(nt, nt, nt), proposal=proposal)
+    assert (lat.get_config() == cfg).all()
+    assert lat.state()[1].tolist() == st.tolist()
+    lat.close()
+
+
+@pytest.mark.parametrize("M,scale,proposal", [(4, 20.0, 0), (4, 20.0, 2), (6, 20.0, 0), (4, 9000.0, 0), (7, 9000.0, 0)])
+def test_batch_lanes_per_trial(M, scale, proposal):
+    # both counter widths and both numbers of byte planes
+    stream = torch.cuda.current_stream()
+    V = epi_gaussian(4, M, scale, 5)
+    dims = [(12, 14, 16), (24, 18, 21), (8, 9, 24)]
+    T = [700.0, 1100.0, 1900.0]
+    lats = []
+    for r, d in enumerate(dims):
+        lat = smcx.Lattice(smcx.BCC, d, M, [1.0 / M] * M, init_seed=30 + r, storage=smcx.INT8, sched=(4, (2, 2, 2)),
+                           stream=stream)
+        lat.set_replica(r)
+        lat.set_epi(V)
+        lat.set_proposal(proposal)
+        lats.append(lat)
+    cfg = [lat.get_config().copy() for lat in lats]
+    b = smcx.Batch(lats, stream)
+    b.sweep(T, 3, 13)
+    for r, d in enumerate(dims):
+        st = O.sweep(O.BCC, d, M, 4, V, cfg[r], T[r], 3, 13, replica=r, L=4, nt=(2, 2, 2), proposal=proposal)
+        assert (lats[r].get_config() == cfg[r]).all()
+        assert lats[r].state()[1].tolist() == st.tolist()
+    b.close()
