@@ -29,6 +29,7 @@ struct smcx_batch {
   int* d_status = nullptr;
   int threads = 0, slots = 1;
   bool group = false;  // several lanes per trial
+  int max_L = 0;       // largest link cell of the replicas
   long long timeout_ns = 2000000000ll;
   int skip_cta = -1;  // fault injection: this CTA never reports its tile pass as done
   bool use_graph = true;
@@ -114,6 +115,7 @@ void rebuild_items(smcx_batch* b) {
   b->group = b->threads != 128 && b->threads != 256 && nq <= 3 && b->n_items <= 2 * kSMs && (!dir || max_L <= 6);
   b->threads = threads;
   b->slots = slots;
+  b->max_L = max_L;
   b->items_proposal = b->lat[0]->proposal;
   for (auto& g : b->graphs) cudaGraphExecDestroy(g.second);
   b->graphs.clear();
@@ -201,7 +203,7 @@ static void batch_sweep_launch(smcx_batch* b, const double* T, int64_t n_sweeps,
   // shared memory for the largest table of this call, rounded up so that a
   // graph instantiated for it serves nearby temperature sets as well
   const int nA_cap = std::min(kNA, ((max_nA + 255) / 256) * 256);
-  const size_t smem = bccfast::smem_bytes(nA_cap);
+  const size_t smem = bccfast::smem_bytes(nA_cap) + (b->lat[0]->proposal != 0 ? bccfast::dir_bytes(b->max_L) : 0);
   check_cuda(cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
              "batch smem attribute");
   int dev = 0, nsm = 0, per_sm = 0;

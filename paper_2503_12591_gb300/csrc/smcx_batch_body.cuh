@@ -96,9 +96,11 @@ __device__ __forceinline__ void batch_body(const Planes& Q, const LatDesc* __res
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ unsigned long long s_stat[3];
   uint32_t* sA = reinterpret_cast<uint32_t*>(smem + 2 * SUB);
+  uint32_t* sB = sA + max_nA;
+  uint8_t* s_dir = reinterpret_cast<uint8_t*>(sB + kNB);
   batch_loop(descs, items, n_items, n_sweeps, pr, status, timeout_ns, skip_cta,
              [&](const LatDesc& D, int tc, int jt, unsigned long long sweep) {
-               bcc_tile_pass<K, NW, PL, SLOTS, PROP>(D, Q, tc, jt, sweep, smem, sA, sA + max_nA, s_stat);
+               bcc_tile_pass<K, NW, PL, SLOTS, PROP>(D, Q, tc, jt, sweep, smem, sA, sB, s_dir, s_stat);
              });
 }
 

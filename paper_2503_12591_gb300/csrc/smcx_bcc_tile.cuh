@@ -415,7 +415,8 @@ __device__ __forceinline__ void finish_trial_rows(uint8_t* box, int s, int sp, u
 // tiles of that colour (plus its 2-cell halo) into shared memory, run every
 // intra-colour phase of the tile, write the tile and its 1-cell partner ring
 // back, add the statistics.  Every thread of the CTA must call it.
-// Shared memory: box (2 * SUB bytes), sA (nA words), sB (kNB words), s_stat[3].
+// Shared memory: box (2 * SUB bytes), sA (nA words), sB (kNB words), s_dir (2 L^3
+// bytes, shared-direction proposals only), s_stat[3].
 // Shared-direction trial; defined where the offset table lives
 // (smcx_sweep_bcc_dir.cu).
 template <int B, int K, int NW, int PL>
@@ -545,8 +546,7 @@ __device__ __forceinline__ void stage_box(const LatDesc& D, uint8_t* box, const 
 template <int K, int NW, int PL, int SLOTS, int PROP = 0, bool TL1 = false>
 __device__ __forceinline__ void bcc_tile_pass(const LatDesc& D, const Planes& Q, int tc, int jt,
                                               unsigned long long sweep, uint8_t* box, uint32_t* sA, uint32_t* sB,
-                                              unsigned long long* s_stat) {
-  __shared__ uint8_t s_dir[512];  // phase directions (shared-direction proposals)
+                                              uint8_t* s_dir, unsigned long long* s_stat) {
   __shared__ __align__(16) uint32_t s_rows[PROP == 1 ? 128 : 4];  // V-difference rows (shared-direction)
   const int tid = threadIdx.x, nth = blockDim.x;
   const int lane = tid & 31, warp = tid >> 5, nwarp = nth >> 5;
@@ -563,7 +563,7 @@ __device__ __forceinline__ void bcc_tile_pass(const LatDesc& D, const Planes& Q,
   // link-cell slots of this thread, in the bank-spreading order where the shape has
   // one.  Shared-direction passes read it before the tile is staged, which hides the
   // load; passes with a direction per trial have no registers to hold it.
-  const int NQ = D.NQ, L = D.L;
+  const int NQ = D.NQ, L = D.L, n_dir = 2 * L * L * L;
   const bool ordered = NQ >= kOrderMinNQ && NQ <= kOrderMaxNQ && L >= kOrderMinL && L <= kOrderMaxL &&
                        nth * SLOTS >= order_lanes(NQ);
   auto slot_of = [&](int j) {
@@ -591,12 +591,12 @@ __device__ __forceinline__ void bcc_tile_pass(const LatDesc& D, const Planes& Q,
     // per (sweep, tile, phase) (mode 1) or per (sweep, colour, block of two
     // tiles, phase) (mode 2)
     const unsigned tile = (unsigned)((ti[2] * D.nt[1] + ti[1]) * D.nt[0] + ti[0]);
-    for (int pr = tid; pr < D.L * D.L * D.L; pr += nth) {
+    for (int pr = tid; pr < n_dir / 2; pr += nth) {
       const uint4 r = D.proposal == 2 ? block_direction_block(D.seed_lo, D.seed_hi, sweep, D.replica, tc,
                                                               (unsigned)jt >> 1, pr)
                                       : phase_direction_block(D.seed_lo, D.seed_hi, sweep, D.replica, tile, pr);
-      st_chk(s_dir, 2 * pr, 512, kDbgBccDir, (uint8_t)(r.x >> 29));
-      st_chk(s_dir, 2 * pr + 1, 512, kDbgBccDir, (uint8_t)(r.z >> 29));
+      st_chk(s_dir, 2 * pr, n_dir, kDbgBccDir, (uint8_t)(r.x >> 29));
+      st_chk(s_dir, 2 * pr + 1, n_dir, kDbgBccDir, (uint8_t)(r.z >> 29));
     }
   }
 
@@ -636,7 +636,7 @@ __device__ __forceinline__ void bcc_tile_pass(const LatDesc& D, const Planes& Q,
             keep_u[j] = rw.w;
             const int s = (zr + h) * PP + (yr + h) * PX + (xr + h);
             if (PROP == 1)
-              trial_shared_dir<0, K, NW, PL>(box, s, ld_chk(s_dir, ((cz * L + cy) * L + cx) * 2, 512, kDbgBccDir),
+              trial_shared_dir<0, K, NW, PL>(box, s, ld_chk(s_dir, ((cz * L + cy) * L + cx) * 2, n_dir, kDbgBccDir),
                                              rw.y, Q, s_rows, D.nA, sA, sB, acc, same, dsum);
             else
               trial<0, K, NW, PL>(box, s, rw.x, rw.y, Q, D.nA, sA, sB, acc, same, dsum);
@@ -650,7 +650,7 @@ __device__ __forceinline__ void bcc_tile_pass(const LatDesc& D, const Planes& Q,
             const int s = (zr + h) * PP + (yr + h) * PX + (xr + h);
             if (PROP == 1)
               trial_shared_dir<1, K, NW, PL>(box, SUB + s,
-                                             ld_chk(s_dir, ((cz * L + cy) * L + cx) * 2 + 1, 512, kDbgBccDir),
+                                             ld_chk(s_dir, ((cz * L + cy) * L + cx) * 2 + 1, n_dir, kDbgBccDir),
                                              keep_u[j], Q, s_rows, D.nA, sA, sB, acc, same, dsum);
             else
               trial<1, K, NW, PL>(box, SUB + s, keep_d[j], keep_u[j], Q, D.nA, sA, sB, acc, same, dsum);
@@ -696,6 +696,11 @@ __device__ __forceinline__ void bcc_tile_pass(const LatDesc& D, const Planes& Q,
 // high-part entries.
 __host__ __device__ constexpr size_t smem_bytes(int nA) { return 2 * SUB + (size_t)(nA + kNB) * 4; }
 
+// Shared-direction proposals: the directions of a pass's 2 L^3 phases, in dynamic shared
+// memory behind the rest (link cells of at most a tile's 20 cells).
+constexpr int kMaxDirL = BOX - 4;
+__host__ __device__ constexpr size_t dir_bytes(int L) { return ((size_t)2 * L * L * L + 15) / 16 * 16; }
+static_assert(2 * SUB % 16 == 0, "directions follow the box");
 
 // Single-lattice sweep kernel: one CTA per tile of colour `tc`.
 template <int K, int NW, int PL, int SLOTS, int PROP>
@@ -705,7 +710,8 @@ __global__ void __launch_bounds__(128, PROP == 1 ? 7 : 6) k_bcc_tile_sweep(const
   uint8_t* box = smem;
   uint32_t* sA = reinterpret_cast<uint32_t*>(smem + 2 * SUB);
   uint32_t* sB = sA + D.nA;
-  bcc_tile_pass<K, NW, PL, SLOTS, PROP, PROP == 1>(D, Q, tc, blockIdx.x, D.sweep, box, sA, sB, s_stat);
+  // shared directions: the tables stay in global memory, s_dir follows the box
+  bcc_tile_pass<K, NW, PL, SLOTS, PROP, PROP == 1>(D, Q, tc, blockIdx.x, D.sweep, box, sA, sB, smem + 2 * SUB, s_stat);
 }
 
 }  // namespace bccfast
@@ -713,7 +719,7 @@ __global__ void __launch_bounds__(128, PROP == 1 ? 7 : 6) k_bcc_tile_sweep(const
 template <int K, int NW, int PL, int SLOTS, int PROP = 0>
 inline void launch_bcc(smcx_lattice* hd, bccfast::LatDesc& D, const bccfast::Planes& Q, int threads,
                        int64_t n_sweeps, int n_colours) {
-  const size_t smem = PROP == 1 ? (size_t)2 * bccfast::SUB : bccfast::smem_bytes(D.nA);
+  const size_t smem = PROP == 1 ? (size_t)2 * bccfast::SUB + bccfast::dir_bytes(D.L) : bccfast::smem_bytes(D.nA);
   check_cuda(cudaFuncSetAttribute(bccfast::k_bcc_tile_sweep<K, NW, PL, SLOTS, PROP>,
                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
              "bcc sweep smem attribute");

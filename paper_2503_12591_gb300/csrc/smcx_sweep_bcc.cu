@@ -47,7 +47,7 @@ bool bcc_fast_usable(const smcx_lattice* hd, int dir_slots) {
   if (hd->kind != kBCC || hd->M > kMaxSweepM || !hd->have_epi) return false;
   if (hd->proposal != 0) {
     // one compiled variant: 4 shells, M <= 4, |V| < 2^15, one slot per thread
-    if (hd->shells.K != 4 || hd->M > 4) return false;
+    if (hd->shells.K != 4 || hd->M > 4 || sc.L > bccfast::kMaxDirL) return false;
     for (int32_t v : hd->V)
       if (v >= 32768 || v <= -32768) return false;
   }

@@ -272,19 +272,24 @@ __host__ __device__ constexpr size_t smem_bytes(int nA) {
   return BOX_BYTES + 16 * 4 + kRowWords * 4 + kPlaneWords * 4 + (size_t)(nA + kNB) * 4;
 }
 
+// Shared-direction proposals: the directions of a pass's 4 L^3 phases follow (link cells
+// of at most a tile's 15 cells).
+__host__ __device__ constexpr size_t dir_bytes(int L) { return ((size_t)4 * L * L * L + 15) / 16 * 16; }
+
 // Five CTAs per SM: the box and its tables (42.8 KB) allow no sixth, so the
 // launch bounds leave the kernel 102 registers (it takes 96).
 template <int K, int NW, int PL, int PROP = 0>
 __global__ void __launch_bounds__(128, 5) k_fcc_tile_sweep(const LatDesc D, const Planes Q, const Rows6 R, int tc) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ unsigned long long s_stat[3];
-  __shared__ uint8_t s_dir[PROP ? 512 : 4];  // phase directions (shared-direction proposals)
   uint8_t* box = smem;
   int* s_poff = reinterpret_cast<int*>(smem + BOX_BYTES);
   int32_t* sR = s_poff + 16;
   uint32_t* sP = reinterpret_cast<uint32_t*>(sR + kRowWords);
   uint32_t* sA = sP + kPlaneWords;
   uint32_t* sB = sA + D.nA;
+  uint8_t* s_dir = reinterpret_cast<uint8_t*>(sB + kNB);  // phase directions (shared-direction proposals)
+  const int n_dir = 4 * D.L * D.L * D.L;
   const int tid = threadIdx.x, nth = blockDim.x;
   const int lane = tid & 31, warp = tid >> 5, nwarp = nth >> 5;
   const int jt = blockIdx.x;
@@ -314,12 +319,12 @@ __global__ void __launch_bounds__(128, 5) k_fcc_tile_sweep(const LatDesc D, cons
     // block of two tiles, ic) (mode 2): one Philox block per ic pair pr =
     // ic >> 1, word 0 for even ic, word 2 for odd ic
     const unsigned tile = (unsigned)((ti[2] * D.nt[1] + ti[1]) * D.nt[0] + ti[0]);
-    for (int pr = tid; pr < 2 * D.L * D.L * D.L; pr += nth) {
+    for (int pr = tid; pr < n_dir / 2; pr += nth) {
       const uint4 r = D.proposal == 2 ? block_direction_block(D.seed_lo, D.seed_hi, D.sweep, D.replica, tc,
                                                               (unsigned)jt >> 1, pr)
                                       : phase_direction_block(D.seed_lo, D.seed_hi, D.sweep, D.replica, tile, pr);
-      st_chk(s_dir, 2 * pr, 512, kDbgBccDir, (uint8_t)__umulhi(r.x, 12u));
-      st_chk(s_dir, 2 * pr + 1, 512, kDbgBccDir, (uint8_t)__umulhi(r.z, 12u));
+      st_chk(s_dir, 2 * pr, n_dir, kDbgBccDir, (uint8_t)__umulhi(r.x, 12u));
+      st_chk(s_dir, 2 * pr + 1, n_dir, kDbgBccDir, (uint8_t)__umulhi(r.z, 12u));
     }
   }
   if (tid < 12) {
@@ -357,7 +362,7 @@ __global__ void __launch_bounds__(128, 5) k_fcc_tile_sweep(const LatDesc D, cons
           if (here) {
             rw = attempt_block(cell * 4 + 2 * pr, D.sweep, D.replica, D.seed_lo, D.seed_hi);
             if constexpr (PROP != 0)
-              trial_dir<K, NW, PL>(box, cbase + boff(2 * pr), ld_chk(s_dir, ic, 512, kDbgBccDir), rw.y, s_poff, sP,
+              trial_dir<K, NW, PL>(box, cbase + boff(2 * pr), ld_chk(s_dir, ic, n_dir, kDbgBccDir), rw.y, s_poff, sP,
                                    sR, D.nA, sA, sB, acc, same, dsum);
             else
               trial<K, NW, PL>(box, cbase + boff(2 * pr), rw.x, rw.y, s_poff, sP, sR, D.nA,
@@ -366,7 +371,7 @@ __global__ void __launch_bounds__(128, 5) k_fcc_tile_sweep(const LatDesc D, cons
           __syncthreads();
           if (here) {
             if constexpr (PROP != 0)
-              trial_dir<K, NW, PL>(box, cbase + boff(2 * pr + 1), ld_chk(s_dir, ic + 1, 512, kDbgBccDir), rw.w,
+              trial_dir<K, NW, PL>(box, cbase + boff(2 * pr + 1), ld_chk(s_dir, ic + 1, n_dir, kDbgBccDir), rw.w,
                                    s_poff, sP, sR, D.nA, sA, sB, acc, same, dsum);
             else
               trial<K, NW, PL>(box, cbase + boff(2 * pr + 1), rw.z, rw.w, s_poff,
@@ -426,7 +431,7 @@ bool fcc_fast_usable(const smcx_lattice* hd) {
   if (hd->kind != kFCC || hd->M > kMaxSweepM || !hd->have_epi || !hd->Wq.empty()) return false;
   if (hd->shells.K > 3) return false;
   if (hd->proposal != SMCX_PROPOSAL_SITE) {
-    if (hd->shells.K != 3 || hd->M > 5) return false;
+    if (hd->shells.K != 3 || hd->M > 5 || sc.L > fccfast::TMAX) return false;
     if (hd->M == 5) {
       // six-bit counters: every field difference fits
     } else {
@@ -491,7 +496,7 @@ void sweep_fcc_fast(smcx_lattice* hd, int nA, uint64_t seed, int64_t n_sweeps, i
           }
         r[15] = (int32_t)(0u - 32u * sum);
       }
-  const size_t smem = fccfast::smem_bytes(nA);
+  const size_t smem = fccfast::smem_bytes(nA) + (D.proposal != 0 ? fccfast::dir_bytes(D.L) : 0);
   const int grid = (D.nt[0] / 2) * (D.nt[1] / 2) * (D.nt[2] / 2);
   auto run = [&](auto kern) {
     check_cuda(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),

@@ -202,3 +202,34 @@ def test_batch_lanes_per_trial(M, scale, proposal):
         assert (lats[r].get_config() == cfg[r]).all()
         assert lats[r].state()[1].tolist() == st.tolist()
     b.close()
+
+
+@pytest.mark.parametrize("kind,L,nt,dims", [(smcx.BCC, 6, 2, (36, 25, 31)), (smcx.BCC, 7, 2, (40, 39, 37)),
+                                            (smcx.BCC, 9, 2, (40, 38, 36)), (smcx.BCC, 18, 2, (40, 39, 37)),
+                                            (smcx.FCC, 5, 2, (30, 27, 23)), (smcx.FCC, 6, 2, (30, 27, 25)),
+                                            (smcx.FCC, 14, 2, (30, 29, 28)), (smcx.FCC, 7, 4, (56, 29, 30))])
+@pytest.mark.parametrize("proposal", [1, 2])
+def test_shared_directions_of_long_link_cells(kind, L, nt, dims, proposal):
+    # 2 L^3 (BCC) or 4 L^3 (FCC) phases a pass, 432 to 11,664 of them
+    M, K = (4, 4) if kind == smcx.BCC else (5, 3)
+    lat, cfg, V = _lattice(kind, dims, M, K, smcx.PACKED4, 33)
+    nts = tuple(nt if n // nt >= L else 2 for n in dims)
+    lat.set_schedule((L, nts))
+    lat.set_proposal(proposal)
+    start = cfg.copy()
+    lat.sweep(1000.0, 2, 37)
+    st = O.sweep(kind, dims, M, K, V, cfg, 1000.0, 2, 37, L=L, nt=nts, proposal=proposal)
+    assert (lat.get_config() == cfg).all()
+    assert lat.state()[1].tolist() == st.tolist()
+    if kind == smcx.BCC:
+        lat2 = smcx.Lattice(kind, dims, M, [0.25] * 4, storage=smcx.PACKED4, sched=(L, nts),
+                            stream=torch.cuda.current_stream())
+        lat2.set_epi(V)
+        lat2.set_config(start)
+        lat2.set_proposal(proposal)
+        b = smcx.Batch([lat2], torch.cuda.current_stream())
+        b.sweep([1000.0], 2, 37)
+        assert (lat2.get_config() == cfg).all()
+        b.close()
+        lat2.close()
+    lat.close()
