@@ -462,94 +462,152 @@ __device__ __forceinline__ const QClass<K>& qclass() {
   if constexpr (K == 2) return TM == 20 ? c_qclass2_20 : c_qclass2_17;
   else return TM == 20 ? c_qclass3_20 : c_qclass3_17;
 }
-// Energy change of the environment-of-s slots [I0, I1): a site holding b
-// (d = +1) or a (d = -1) sees its count in the shell of s move by d and in
-// the shell of s' (if any) by -d; a count n moving by d changes the term by
-// W (2 n d + d^2); other species give d = 0.
+// Sums over changing sites of one species, per shell: the counts n_k of the sites that
+// gain (g) and that lose (l) a same-species neighbour in shell k, as masked words (n_k
+// << fshift(k), 50 sites of at most 24 << 10 in all) with the number of sites from
+// bit 24 on.  One masked word and one add per site and shell; the weights come once at the end.
+template <int K>
+struct CountSums {
+  uint32_t g[K], l[K];
+  __device__ __forceinline__ CountSums() {
+#pragma unroll
+    for (int k = 0; k < K; k++) g[k] = l[k] = 0;
+  }
+  // sum_k W[k] (n' ^ 2 - n^2) over these sites: 2 n + 1 for a gain, 1 - 2 n for a loss
+  __device__ __forceinline__ int energy(const int (&wq)[K]) const {
+    int dE = 0;
+#pragma unroll
+    for (int k = 0; k < K; k++) {
+      const int ng = (int)((g[k] & 0xFFFFFFu) >> fshift(k)), nl = (int)((l[k] & 0xFFFFFFu) >> fshift(k));
+      dE += wq[k] * (2 * (ng - nl) + (int)((g[k] >> 24) + (l[k] >> 24)));
+    }
+    return dE;
+  }
+};
+template <int K>
+__device__ __forceinline__ uint32_t counted(uint32_t w, int k) {
+  return (w & ((uint32_t)fmask(k) << fshift(k))) | (1u << 24);
+}
+// The environment-of-s slots [I0, I1) after the swap: a site holding b gains a
+// neighbour in the shell of s and loses one in the shell of s' (if any), a site
+// holding a the reverse.
 template <int K, int TM, int I0, int I1>
-__device__ __forceinline__ int es_energy(const uint16_t* box, const short* es, int s, int sa, int sb,
-                                         const int (&wqa)[K], const int (&wqb)[K]) {
+__device__ __forceinline__ void es_sums(const uint16_t* box, const short* es, int s, int sa, int sb, CountSums<K>& A,
+                                        CountSums<K>& B) {
   constexpr QClass<K> QC = make_qclass<K, TM>();
-  int dE = 0;
 #pragma unroll
   for (int i = I0; i < I1; i++) {
     const uint32_t w = box[s + es[i]];
     const int c = (int)(w & 7u);
-    const bool isb = c == sb, isa = c == sa;
-    const int d = (int)isb - (int)isa, ad = (int)(isb | isa);
     const int k1 = QC.k1[i], k2 = QC.k2[i];
-    const int n1 = (int)((w >> fshift(k1)) & (uint32_t)fmask(k1));
-    dE += (isb ? wqb[k1] : wqa[k1]) * (2 * d * n1 + ad);
-    if (k2 >= 0) {
-      const int n2 = (int)((w >> fshift(k2)) & (uint32_t)fmask(k2));
-      dE += (isb ? wqb[k2] : wqa[k2]) * (ad - 2 * d * n2);
+    const uint32_t x1 = counted<K>(w, k1), x2 = k2 >= 0 ? counted<K>(w, k2 >= 0 ? k2 : 0) : 0;
+    if (c == sb) {
+      B.g[k1] += x1;
+      if (k2 >= 0) B.l[k2 >= 0 ? k2 : 0] += x2;
+    }
+    if (c == sa) {
+      A.l[k1] += x1;
+      if (k2 >= 0) A.g[k2 >= 0 ? k2 : 0] += x2;
     }
   }
-  return dE;
 }
-// The count updates of the same slots after an accepted swap.
+// The count updates of the same slots after an accepted swap.  The words of a group of
+// slots are loaded before any is stored (a store in between holds the next load back:
+// it might be to the same word), and all are stored, changed or not: no other trial of
+// a phase has a slot of this one.  120^3 cells, 5 species, 3 shells, with the sums
+// above: 8.2 -> 5.9 ms per sweep; 320^3 23.3 -> 18.1; 120^3 with two shells 4.5 -> 3.1.
+constexpr int kUpdateGroup = 20;
 template <int K, int TM, int I0, int I1>
 __device__ __forceinline__ void es_update(uint16_t* box, const short* es, int s, int sa, int sb) {
   constexpr QClass<K> QC = make_qclass<K, TM>();
 #pragma unroll
-  for (int i = I0; i < I1; i++) {
-    const int t = s + es[i];
-    const uint32_t w = box[t];
-    const int c = (int)(w & 7u);
-    const int d = (int)(c == sb) - (int)(c == sa);
-    const int k1 = QC.k1[i], k2 = QC.k2[i];
-    const int dw = d * ((1 << fshift(k1)) - (k2 >= 0 ? (1 << fshift(k2)) : 0));
-    if (d != 0) box[t] = (uint16_t)((int)w + dw);
+  for (int g = I0; g < I1; g += kUpdateGroup) {
+    int t[kUpdateGroup];
+    uint32_t w[kUpdateGroup];
+#pragma unroll
+    for (int i = 0; i < kUpdateGroup; i++)
+      if (g + i < I1) {
+        t[i] = s + es[g + i];
+        w[i] = box[t[i]];
+      }
+#pragma unroll
+    for (int i = 0; i < kUpdateGroup; i++)
+      if (g + i < I1) {
+        const int c = (int)(w[i] & 7u);
+        const int k1 = QC.k1[g + i], k2 = QC.k2[g + i];
+        const int d = (int)(c == sb) - (int)(c == sa);
+        const int dw = d * ((1 << fshift(k1)) - (k2 >= 0 ? (1 << fshift(k2)) : 0));
+        box[t[i]] = (uint16_t)((int)w[i] + dw);
+      }
   }
 }
-// Sites around s' outside the environment of s: a site holding a (d = +1)
-// or b (d = -1) sees its count in the shell of s' move by d.
+// Sites around s' outside the environment of s: a site holding a gains a neighbour in
+// the shell of s', a site holding b loses one.
 template <int K, int TM>
-__device__ __forceinline__ int ep_energy(const uint16_t* box, const short* ep, int sp, int sa, int sb,
-                                         const int (&wqa)[K], const int (&wqb)[K]) {
+__device__ __forceinline__ void ep_sums(const uint16_t* box, const short* ep, int sp, int sa, int sb, CountSums<K>& A,
+                                        CountSums<K>& B) {
   constexpr QClass<K> QC = make_qclass<K, TM>();
-  int dE = 0;
 #pragma unroll
   for (int i = 0; i < QC.NP; i++) {
     const uint32_t w = box[sp + ep[i]];
     const int c = (int)(w & 7u);
-    const bool isb = c == sb, isa = c == sa;
-    const int d = (int)isa - (int)isb, ad = (int)(isb | isa);
     const int k = QC.kp[i];
-    const int n = (int)((w >> fshift(k)) & (uint32_t)fmask(k));
-    dE += (isb ? wqb[k] : wqa[k]) * (2 * d * n + ad);
+    const uint32_t x = counted<K>(w, k);
+    if (c == sa) A.g[k] += x;
+    if (c == sb) B.l[k] += x;
   }
-  return dE;
 }
-template <int K, int TM>
+template <int K, int TM, int I0, int I1>
 __device__ __forceinline__ void ep_update(uint16_t* box, const short* ep, int sp, int sa, int sb) {
   constexpr QClass<K> QC = make_qclass<K, TM>();
 #pragma unroll
-  for (int i = 0; i < QC.NP; i++) {
-    const int t = sp + ep[i];
-    const uint32_t w = box[t];
-    const int c = (int)(w & 7u);
-    const int d = (int)(c == sa) - (int)(c == sb);
-    if (d != 0) box[t] = (uint16_t)((int)w + d * (1 << fshift(QC.kp[i])));
+  for (int g = I0; g < I1; g += kUpdateGroup) {
+    int t[kUpdateGroup];
+    uint32_t w[kUpdateGroup];
+#pragma unroll
+    for (int i = 0; i < kUpdateGroup; i++)
+      if (g + i < I1) {
+        t[i] = sp + ep[g + i];
+        w[i] = box[t[i]];
+      }
+#pragma unroll
+    for (int i = 0; i < kUpdateGroup; i++)
+      if (g + i < I1) {
+        const int c = (int)(w[i] & 7u);
+        const int d = (int)(c == sa) - (int)(c == sb);
+        box[t[i]] = (uint16_t)((int)w[i] + d * (1 << fshift(QC.kp[g + i])));
+      }
   }
 }
-// Pair part around one end: sum_k sum_v W[k][c(e + v)] (SIGN +1 around s,
-// -1 around s'), with the counts of species a and b there.
+// Pair part around one end: sum_k sum_v W[k][c(e + v)] (SIGN +1 around s, -1 around
+// s'), with the counts n of species `sc` there (of the end's own species the box
+// holds them).
 template <int K, int TM, int SIGN>
-__device__ __forceinline__ int pair_side(const uint16_t* box, int e, const int32_t* W, int M, int sa, int sb,
-                                         int (&na)[K], int (&nb)[K]) {
+__device__ __forceinline__ int pair_side(const uint16_t* box, int e, const int32_t* W, int M, int sc, int (&n)[K]) {
   constexpr qfcc::QTable T = qfcc::make_qvecs();
   constexpr int NV = vec_count(kFCC, K);
   int dE = 0;
 #pragma unroll
-  for (int k = 0; k < K; k++) na[k] = nb[k] = 0;
+  for (int k = 0; k < K; k++) n[k] = 0;
 #pragma unroll
   for (int j = 0; j < NV; j++) {
     const int k = T.v[j].k;
     const int c = box[e + QBox<TM>::voff(T.v[j].x, T.v[j].y, T.v[j].z)] & 7;
     dE += SIGN * W[k * M + c];
-    na[k] += (c == sa);
-    nb[k] += (c == sb);
+    n[k] += (c == sc);
+  }
+  return dE;
+}
+// Quadratic terms of s and s': b around s (nb) and a around s' (na) after the swap, the
+// counts in their words ws and wp before.
+template <int K>
+__device__ __forceinline__ int own_energy(uint32_t ws, uint32_t wp, const int (&nb)[K], const int (&na)[K],
+                                          const int (&wqa)[K], const int (&wqb)[K]) {
+  int dE = 0;
+#pragma unroll
+  for (int k = 0; k < K; k++) {
+    const int as = field_rt(ws, k), bp = field_rt(wp, k);
+    dE += wqb[k] * (nb[k] * nb[k] - bp * bp) + wqa[k] * (na[k] * na[k] - as * as);
   }
   return dE;
 }
@@ -783,7 +841,8 @@ __global__ void __launch_bounds__(128, TM == 20 ? 2 : 3)
             const int s = cbase + BX::voff(bx_of(b), by_of(b), bz_of(b));
             const int dir = (int)__umulhi(rd, 12u);
             const int sp = s + S.qoff[dir];
-            const int sa = box[s] & 7, sb = box[sp] & 7;
+            const uint32_t ws = box[s], wp = box[sp];
+            const int sa = (int)(ws & 7u), sb = (int)(wp & 7u);
             if (sa == sb) {
               same++;
             } else {
@@ -794,27 +853,26 @@ __global__ void __launch_bounds__(128, TM == 20 ? 2 : 3)
                 wqa[k] = S.wq[k * M + sa];
                 wqb[k] = S.wq[k * M + sb];
               }
-              // pair part and the counts of s and s' after the swap: b
-              // around s without s' (which holds b before the swap), a around
-              // s' without s
-              int na_s[K], nb_s[K], na_p[K], nb_p[K];
-              int dE = s_w[MM * KM + sa * M + sb] + pair_side<K, TM, 1>(box, s, W, M, sa, sb, na_s, nb_s) +
-                       pair_side<K, TM, -1>(box, sp, W, M, sa, sb, na_p, nb_p);
+              // pair part and the counts of s and s' after the swap: b around s without
+              // s' (which holds b before the swap), a around s' without s
+              int nb_s[K], na_p[K];
+              int dE = s_w[MM * KM + sa * M + sb] + pair_side<K, TM, 1>(box, s, W, M, sb, nb_s) +
+                       pair_side<K, TM, -1>(box, sp, W, M, sa, na_p);
               nb_s[0]--;
               na_p[0]--;
-#pragma unroll
-              for (int k = 0; k < K; k++)
-                dE += wqb[k] * (nb_s[k] * nb_s[k] - nb_p[k] * nb_p[k]) + wqa[k] * (na_p[k] * na_p[k] - na_s[k] * na_s[k]);
+              dE += own_energy<K>(ws, wp, nb_s, na_p, wqa, wqb);
               // environment sites whose counts move
               const short* es = S.es + dir * S.NS;
               const short* ep = S.ep + dir * S.NP;
-              dE += es_energy<K, TM, 0, Tables<K, TM>::NS>(box, es, s, sa, sb, wqa, wqb);
-              dE += ep_energy<K, TM>(box, ep, sp, sa, sb, wqa, wqb);
+              CountSums<K> A, B;
+              es_sums<K, TM, 0, Tables<K, TM>::NS>(box, es, s, sa, sb, A, B);
+              ep_sums<K, TM>(box, ep, sp, sa, sb, A, B);
+              dE += A.energy(wqa) + B.energy(wqb);
               if (metropolis_accept(dE, ru, P.thr, P.nA, P.thr + kNA)) {
                 box[s] = (uint16_t)(sb | (pack_counts<K>(nb_s) << 3));
                 box[sp] = (uint16_t)(sa | (pack_counts<K>(na_p) << 3));
                 es_update<K, TM, 0, Tables<K, TM>::NS>(box, es, s, sa, sb);
-                ep_update<K, TM>(box, ep, sp, sa, sb);
+                ep_update<K, TM, 0, Tables<K, TM>::NP>(box, ep, sp, sa, sb);
                 acc++;
                 dsum += dE;
               }
@@ -834,9 +892,11 @@ __global__ void __launch_bounds__(128, TM == 20 ? 2 : 3)
 // counts of s and s') in shared memory, meet at a barrier, and each decides for
 // itself and makes the updates of its own sites; role 1 draws the next words.
 // For lattices with at most one tile of a colour per SM, whose sweep is a chain of
-// 2,048 phases: 120^3 cells, 5 species, 3 shells 10.5 -> 8.3 ms per sweep, 64^3
-// 11.2 -> 7.5, 200^3 11.5 -> 8.5.  With more tiles the SMs have warps enough and
-// k_qsro_fcc_n's fewer instructions win (320^3 in 16-cell tiles: 31.1 against 40.8).
+// 2,048 phases (5 species, 3 shells, L = 4, ms per sweep, one thread and four): 24^3
+// cells 5.14 and 3.81, 64^3 5.26 and 4.19, 160^3 in 16-cell tiles 5.32 and 4.76, 120^3
+// and 200^3 (20-cell tiles) 6.11 and 5.87, 6.20 and 5.93.  With more tiles the SMs have
+// warps enough and k_qsro_fcc_n's fewer instructions win (240^3 9.06 against 10.22,
+// 320^3 18.1 against 20.3), with two shells nearly always (120^3 3.13 against 3.74).
 constexpr int kQsroSlots = 128;     // link-cell slots of a tile at most
 constexpr int kQsroRoles = 4;
 template <int K, int TM>
@@ -847,10 +907,14 @@ __global__ void __launch_bounds__(kQsroSlots * kQsroRoles)
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ Tables<K, TM> S;
   constexpr int NS = Tables<K, TM>::NS;
-  constexpr int NSA = NS * 20 / 33;  // environment-of-s sites of role 2; role 3 takes the rest and ep
+  constexpr int NP = Tables<K, TM>::NP;
+  // updates: es [0, U0), es [U0, U1), es [U1, NS) and ep [0, U2), ep [U2, NP)
+  constexpr int U0 = (NS + NP) * 2 / 7, U1 = U0 + (NS + NP) / 7, U2 = NP - (NS + NP) * 2 / 7;
+  static_assert(0 < U0 && U1 <= NS && 0 <= U2, "shares of the updates");
+  constexpr int NSA = NS * 22 / 33;  // environment-of-s sites of role 2; role 3 takes the rest and ep
   __shared__ uint4 s_rw[kQsroSlots];              // Philox block of the slot's site pair
   __shared__ int s_part[kQsroRoles][kQsroSlots];  // shares of dE
-  __shared__ int s_cnt[2][kQsroSlots][K];         // counts around s and s': a | b << 8
+  __shared__ int s_cnt[2][kQsroSlots][K];         // b around s, a around s' after the swap
   const int tid = threadIdx.x;
   const int M = P.M, KM = K * P.M, MM = P.M * P.M;
   uint16_t* box = reinterpret_cast<uint16_t*>(smem);
@@ -865,7 +929,9 @@ __global__ void __launch_bounds__(kQsroSlots * kQsroRoles)
   long long dsum = 0;
   const int L = P.L;
   const int NQ = (max(ts[0], max(ts[1], ts[2])) + L - 1) / L;
-  const int role = tid / kQsroSlots, sl = tid % kQsroSlots;
+  // A warp of each role for 32 slots in every group of four warps, which the hardware
+  // spreads over the SM's four schedulers; the role rotates from group to group.
+  const int role = ((tid >> 5) + (tid >> 7)) & 3, sl = (tid >> 7) * 32 + (tid & 31);
   const int qx = sl % NQ, qy = (sl / NQ) % NQ, qz = sl / (NQ * NQ);
   const bool slot = sl < NQ * NQ * NQ;
   // random words of site pair pr (sublattices 2 pr, 2 pr + 1) of the slot's cell
@@ -886,15 +952,17 @@ __global__ void __launch_bounds__(kQsroSlots * kQsroRoles)
         const int cbase = BX::eidx(2 * xr + 3, 2 * yr + 3, 2 * zr + 3);
         for (int b = 0; b < 4; b++) {
           int s = 0, sp = 0, sa = 0, sb = 0, dir = 0;
-          uint32_t ru = 0;
+          uint32_t ru = 0, ws = 0, wp = 0;
           if (here) {
             const uint4 rw = s_rw[sl];
             ru = (b & 1) ? rw.w : rw.y;
             dir = (int)__umulhi((b & 1) ? rw.z : rw.x, 12u);
             s = cbase + BX::voff(bx_of(b), by_of(b), bz_of(b));
             sp = s + S.qoff[dir];
-            sa = box[s] & 7;
-            sb = box[sp] & 7;
+            ws = box[s];
+            wp = box[sp];
+            sa = (int)(ws & 7u);
+            sb = (int)(wp & 7u);
           }
           const bool live = here && sa != sb;
           if (here && !live && role == 0) same++;
@@ -904,16 +972,12 @@ __global__ void __launch_bounds__(kQsroSlots * kQsroRoles)
             const int32_t* W = s_w + (sa * M + sb) * KM;
             int part;
             if (role < 2) {
-              int na[K], nb[K];
-              if (role == 0) {
-                part = s_w[MM * KM + sa * M + sb] + pair_side<K, TM, 1>(box, s, W, M, sa, sb, na, nb);
-                nb[0]--;  // s' holds b before the swap
-              } else {
-                part = pair_side<K, TM, -1>(box, sp, W, M, sa, sb, na, nb);
-                na[0]--;  // s holds a before the swap
-              }
+              int n[K];
+              if (role == 0) part = s_w[MM * KM + sa * M + sb] + pair_side<K, TM, 1>(box, s, W, M, sb, n);
+              else part = pair_side<K, TM, -1>(box, sp, W, M, sa, n);
+              n[0]--;  // before the swap s' holds b, s holds a
 #pragma unroll
-              for (int k = 0; k < K; k++) s_cnt[role][sl][k] = na[k] | (nb[k] << 8);
+              for (int k = 0; k < K; k++) s_cnt[role][sl][k] = n[k];
             } else {
               int wqa[K], wqb[K];
 #pragma unroll
@@ -921,11 +985,14 @@ __global__ void __launch_bounds__(kQsroSlots * kQsroRoles)
                 wqa[k] = S.wq[k * M + sa];
                 wqb[k] = S.wq[k * M + sb];
               }
-              if (role == 2)
-                part = es_energy<K, TM, 0, NSA>(box, es, s, sa, sb, wqa, wqb);
-              else
-                part = es_energy<K, TM, NSA, NS>(box, es, s, sa, sb, wqa, wqb) +
-                       ep_energy<K, TM>(box, ep, sp, sa, sb, wqa, wqb);
+              CountSums<K> A, B;
+              if (role == 2) {
+                es_sums<K, TM, 0, NSA>(box, es, s, sa, sb, A, B);
+              } else {
+                es_sums<K, TM, NSA, NS>(box, es, s, sa, sb, A, B);
+                ep_sums<K, TM>(box, ep, sp, sa, sb, A, B);
+              }
+              part = A.energy(wqa) + B.energy(wqb);
             }
             s_part[role][sl] = part;
           }
@@ -934,28 +1001,30 @@ __global__ void __launch_bounds__(kQsroSlots * kQsroRoles)
             // every role: the whole dE, with the quadratic terms of s and s' from
             // the counts they have before (a at s, b at s') and after the swap
             int dE = (s_part[0][sl] + s_part[1][sl]) + (s_part[2][sl] + s_part[3][sl]);
-            int nb_s[K], na_p[K];
+            int nb_s[K], na_p[K], wqa[K], wqb[K];
 #pragma unroll
             for (int k = 0; k < K; k++) {
-              const int cs = s_cnt[0][sl][k], cp = s_cnt[1][sl][k];
-              const int na_s = cs & 255, nb_p = cp >> 8;
-              nb_s[k] = cs >> 8;
-              na_p[k] = cp & 255;
-              dE += S.wq[k * M + sb] * (nb_s[k] * nb_s[k] - nb_p * nb_p) +
-                    S.wq[k * M + sa] * (na_p[k] * na_p[k] - na_s * na_s);
+              nb_s[k] = s_cnt[0][sl][k];
+              na_p[k] = s_cnt[1][sl][k];
+              wqa[k] = S.wq[k * M + sa];
+              wqb[k] = S.wq[k * M + sb];
             }
+            dE += own_energy<K>(ws, wp, nb_s, na_p, wqa, wqb);
             if (metropolis_accept(dE, ru, P.thr, P.nA, P.thr + kNA)) {
+              // the four roles share the updates; role 1 also draws words
               if (role == 0) {
                 box[s] = (uint16_t)(sb | (pack_counts<K>(nb_s) << 3));
+                es_update<K, TM, 0, U0>(box, es, s, sa, sb);
                 acc++;
                 dsum += dE;
               } else if (role == 1) {
                 box[sp] = (uint16_t)(sa | (pack_counts<K>(na_p) << 3));
+                es_update<K, TM, U0, U1>(box, es, s, sa, sb);
               } else if (role == 2) {
-                es_update<K, TM, 0, NSA>(box, es, s, sa, sb);
+                es_update<K, TM, U1, NS>(box, es, s, sa, sb);
+                ep_update<K, TM, 0, U2>(box, ep, sp, sa, sb);
               } else {
-                es_update<K, TM, NSA, NS>(box, es, s, sa, sb);
-                ep_update<K, TM>(box, ep, sp, sa, sb);
+                ep_update<K, TM, U2, NP>(box, ep, sp, sa, sb);
               }
             }
           }
@@ -1175,14 +1244,12 @@ void sweep_qsro_device(smcx_lattice* hd, int nA, uint64_t seed, int64_t n_sweeps
     const bool small = tm <= 17;  // the 66 KB box: three CTAs per SM
     const size_t smem = (small ? qfn::QBox<17>::BOX_BYTES : qfn::QBox<20>::BOX_BYTES) + (size_t)nW * 4;
     const int grid = P.ntc[0] * P.ntc[1] * P.ntc[2];
-    // four threads per trial while a colour has at most one tile per SM (measured
-    // at k_qsro_fcc_roles)
-    const bool roles = grid <= kSMs;
+    // three shells: four threads per trial while a colour has at most one tile per SM
+    // (measured at k_qsro_fcc_roles); two shells, half the work, gain nothing from it
+    const bool roles = K == 3 && grid <= kSMs;
     auto kern = K == 2 ? (small ? k_qsro_fcc_n<2, 17> : k_qsro_fcc_n<2, 20>)
                        : (small ? k_qsro_fcc_n<3, 17> : k_qsro_fcc_n<3, 20>);
-    if (roles)
-      kern = K == 2 ? (small ? k_qsro_fcc_roles<2, 17> : k_qsro_fcc_roles<2, 20>)
-                    : (small ? k_qsro_fcc_roles<3, 17> : k_qsro_fcc_roles<3, 20>);
+    if (roles) kern = small ? k_qsro_fcc_roles<3, 17> : k_qsro_fcc_roles<3, 20>;
     const int threads = roles ? kQsroSlots * kQsroRoles : 128;
     check_cuda(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
                "qSRO FCC smem attribute");
