@@ -62,6 +62,9 @@ __device__ __forceinline__ void pair_counts_tile(const LatDesc& D, int t, unsign
     for (int B = 0; B < 2; B++) {
       const int s = s0 + B * SUB;
       const int p = box[s] >> 3;
+      uint32_t is_p[4];
+#pragma unroll
+      for (int pp = 0; pp < 4; pp++) is_p[pp] = p == pp;
       uint32_t hk[K];
 #pragma unroll
       for (int k = 0; k < K; k++) hk[k] = 0;
@@ -77,11 +80,10 @@ __device__ __forceinline__ void pair_counts_tile(const LatDesc& D, int t, unsign
       for (int k = 0; k < K; k++) {
         const uint32_t lo = hk[k] & 0x00FF00FFu, hi = (hk[k] >> 8) & 0x00FF00FFu;
 #pragma unroll
-        for (int pp = 0; pp < 4; pp++)
-          if (p == pp) {
-            acc[k][pp][0] += lo;
-            acc[k][pp][1] += hi;
-          }
+        for (int pp = 0; pp < 4; pp++) {
+          add_if(acc[k][pp][0], lo, is_p[pp]);
+          add_if(acc[k][pp][1], hi, is_p[pp]);
+        }
       }
     }
   }
@@ -109,8 +111,12 @@ __device__ __forceinline__ void pair_counts_tile(const LatDesc& D, int t, unsign
   }
 }
 
+// Four CTAs per SM, 64 registers: the loads of the staging spill some, the loop over
+// the cells does not.  256^3 cells, 4 species, 4 shells: with branches on the species
+// and two CTAs per SM 477 us, without branches 332, with four CTAs 256; 64 lattices of
+// 48^3 cells 227 -> 128; the energy 248 -> 190.
 template <int K>
-__global__ void __launch_bounds__(256) k_bcc_pair_counts(const LatDesc D, unsigned long long* __restrict__ counts) {
+__global__ void __launch_bounds__(256, 4) k_bcc_pair_counts(const LatDesc D, unsigned long long* __restrict__ counts) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ unsigned int hist[kMaxShells * 16];
   pair_counts_tile<K>(D, blockIdx.x, counts, smem, hist);
@@ -119,7 +125,7 @@ __global__ void __launch_bounds__(256) k_bcc_pair_counts(const LatDesc D, unsign
 // Many lattices in one launch: CTA i takes tile items[i].y of lattice
 // items[i].x and adds into counts + items[i].x * kmm.
 template <int K>
-__global__ void __launch_bounds__(256) k_bcc_pair_counts_multi(const LatDesc* __restrict__ descs,
+__global__ void __launch_bounds__(256, 4) k_bcc_pair_counts_multi(const LatDesc* __restrict__ descs,
                                                               const int2* __restrict__ items, int kmm,
                                                               unsigned long long* __restrict__ counts) {
   extern __shared__ __align__(16) unsigned char smem[];
@@ -136,7 +142,7 @@ __global__ void __launch_bounds__(256) k_bcc_pair_counts_multi(const LatDesc* __
 // over the byte planes of V (two or three planes, |V| < 2^23), the rows read
 // from a shared table indexed by the site's species.
 template <int K, int PL>
-__global__ void __launch_bounds__(256) k_bcc_energy(const LatDesc D, const Planes Q, long long* __restrict__ E) {
+__global__ void __launch_bounds__(256, 4) k_bcc_energy(const LatDesc D, const Planes Q, long long* __restrict__ E) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ uint32_t sP[PL * kMaxShells * 4];
   __shared__ long long part[8];

@@ -43,6 +43,12 @@ struct CellIndex {
   }
 };
 
+// acc += x * one (one: 0 or 1), without the branch that the compiler makes of a test of
+// the lane's species: where lanes differ, it runs every branch in turn.
+__device__ __forceinline__ void add_if(uint32_t& acc, uint32_t x, uint32_t one) {
+  asm("mad.lo.u32 %0, %1, %2, %0;" : "+r"(acc) : "r"(x), "r"(one));
+}
+
 }  // namespace bccfast
 
 }  // namespace smcx
