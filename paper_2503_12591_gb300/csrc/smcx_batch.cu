@@ -27,6 +27,8 @@ struct smcx_batch {
   int n_items = 0;
   smcx::bccfast::Progress* d_progress = nullptr;
   int* d_status = nullptr;
+  int block = 0;  // threads per CTA that the caller set: 128 or 256, 0 for the library's choice
+  // the block shape of the work list, made anew with it from `block`
   int threads = 0, slots = 1;
   bool group = false;  // several lanes per trial
   int max_L = 0;       // largest link cell of the replicas
@@ -101,19 +103,19 @@ void rebuild_items(smcx_batch* b) {
   // shared-direction proposals run one slot per thread: tiles of more than
   // 128 slots take 256-thread CTAs unless 128 threads were asked for
   const bool dir = b->lat[0]->proposal != 0;
-  if (b->threads == 256 || (dir && b->threads != 128 && nq * nq * nq > 128)) {
+  if (b->block == 256 || (dir && b->block != 128 && nq * nq * nq > 128)) {
     threads = 256;  // one slot per thread
     slots = 1;
     if (nq * nq * nq > 256) fail(SMCX_E_UNSUPPORTED, "256-thread CTAs take tiles of at most 256 link-cell slots");
   } else {
-    bcc_block_shape(nq, b->threads, &threads, &slots);
+    bcc_block_shape(nq, b->block, &threads, &slots);
   }
   if (slots > 2) fail(SMCX_E_UNSUPPORTED, "batched tiles need at most 256 link-cell slots");
   // Four lanes per trial while a colour has at most two tiles per SM and no tile has
   // more than 3^3 slots: 216 tiles 0.443 -> 0.362 ms a sweep, 343 tiles 0.894 -> 0.907.
   // A block size that was set is kept.
-  b->group = b->threads != 128 && b->threads != 256 && nq <= 3 && b->n_items <= 2 * kSMs && (!dir || max_L <= 6);
-  b->threads = threads;
+  b->group = b->block == 0 && nq <= 3 && b->n_items <= 2 * kSMs && (!dir || max_L <= 6);
+  b->threads = b->group ? bccfast::kGroupThreads : threads;
   b->slots = slots;
   b->max_L = max_L;
   b->items_proposal = b->lat[0]->proposal;
@@ -199,7 +201,7 @@ static void batch_sweep_launch(smcx_batch* b, const double* T, int64_t n_sweeps,
   const int nw = b->lat[0]->M <= 4 ? 1 : 2;
   BatchKernelFn fn =
       b->group ? batch_group_kernel(nw, PL) : pick_kernel(nw, PL, b->slots, b->threads, b->lat[0]->proposal);
-  const int threads = b->group ? bccfast::kGroupThreads : b->threads;
+  const int threads = b->threads;
   // shared memory for the largest table of this call, rounded up so that a
   // graph instantiated for it serves nearby temperature sets as well
   const int nA_cap = std::min(kNA, ((max_nA + 255) / 256) * 256);
@@ -296,6 +298,7 @@ void batch_autotune(smcx_batch* b, const double* T, int trial, int* best_threads
     unsigned long long stats[4];
   };
   std::vector<Saved> saved(R);
+  const int block0 = b->block;
   for (size_t r = 0; r < R; r++) {
     smcx_lattice* h = b->lat[r];
     check_cuda(cudaMalloc(&saved[r].d_copy, h->site_bytes), "autotune snapshot");
@@ -338,7 +341,7 @@ void batch_autotune(smcx_batch* b, const double* T, int trial, int* best_threads
     }
     if (!ok) continue;
     for (size_t r = 0; r < R; r++) b->lat[r]->sched = sc[r];
-    b->threads = c.threads;
+    b->block = c.threads;
     b->items_dirty = true;
     bool usable = true;
     for (size_t r = 0; r < R; r++) usable = usable && bcc_fast_usable(b->lat[r], 256);
@@ -381,9 +384,9 @@ void batch_autotune(smcx_batch* b, const double* T, int trial, int* best_threads
   }
   check_cuda(cudaStreamSynchronize(b->stream), "autotune restore sync");
   for (auto& s : saved) cudaFree(s.d_copy);
-  if (best >= 1e300) fail(SMCX_E_SCHEDULE, "no autotuner candidate fits these lattices");
-  b->threads = bestc.threads;
+  b->block = b->threads = best < 1e300 ? bestc.threads : block0;
   b->items_dirty = true;
+  if (best >= 1e300) fail(SMCX_E_SCHEDULE, "no autotuner candidate fits these lattices");
   if (best_threads) *best_threads = bestc.threads;
 }
 
@@ -605,7 +608,7 @@ int smcx_batch_info(const smcx_batch* b, int* grid, int* threads, int* used_grap
   return guarded_call([&] {
     need_(b != nullptr, SMCX_E_INVALID_ARG, "NULL batch");
     if (grid) *grid = b->last_grid;
-    if (threads) *threads = b->group ? bccfast::kGroupThreads : b->threads;
+    if (threads) *threads = b->threads;
     if (used_graph) *used_graph = b->last_graph ? 1 : 0;
   });
 }
@@ -614,7 +617,7 @@ int smcx_batch_set_block(smcx_batch* b, int threads) {
   return guarded_call([&] {
     need_(b != nullptr, SMCX_E_INVALID_ARG, "NULL batch");
     need_(threads == 0 || threads == 128 || threads == 256, SMCX_E_INVALID_ARG, "threads must be 0, 128 or 256");
-    b->threads = threads;
+    b->block = b->threads = threads;
     b->items_dirty = true;
   });
 }

@@ -162,6 +162,32 @@ def test_batch_shared_direction_equals_plain_and_oracle(stream, mode, threads):
         l.close()
 
 
+def test_batch_proposal_modes_in_turn(stream):
+    """A batch of 6^3-slot tiles without a set block size goes from a direction
+    per trial (two slots per thread) to shared directions (256 threads) and
+    back: the shape of one mode is not the caller's wish for the next."""
+    dims = [(36, 34, 32), (18, 18, 18)]
+    V = epi_gaussian(4, 4, 20.0, 29)
+    T = log_temperatures(len(dims), 500.0, 2500.0)
+    scheds = [_sched(d, L=3, target=18) for d in dims]
+    lats = [_make(d, r, V, stream, scheds[r]) for r, d in enumerate(dims)]
+    b = smcx.Batch(lats, stream)
+    cfg = [O.init_config(O.BCC, d, 4, [0.25] * 4, 100 + r) for r, d in enumerate(dims)]
+    for n, (mode, threads) in enumerate([(smcx.PROPOSAL_SITE, 128), (smcx.PROPOSAL_TILE, 256),
+                                         (smcx.PROPOSAL_SITE, 128), (smcx.PROPOSAL_BLOCK, 256)]):
+        for l in lats:
+            l.set_proposal(mode)
+        b.sweep(T, 1, 47)
+        assert b.info()["threads"] == threads
+        for r, d in enumerate(dims):
+            O.sweep(O.BCC, d, 4, 4, V, cfg[r], T[r], 1, 47, sweep0=n, replica=r, L=scheds[r][0], nt=scheds[r][1],
+                    proposal=mode)
+            assert (lats[r].get_config() == cfg[r]).all(), f"replica {r}, mode {mode}"
+    b.close()
+    for l in lats:
+        l.close()
+
+
 def test_batch_mixed_proposal_modes_refused(stream):
     V = epi_gaussian(4, 4, 20.0, 1)
     dims = [(12, 12, 12), (16, 16, 16)]
