@@ -39,6 +39,7 @@ struct smcx_batch {
   std::vector<int32_t> graph_V;                 // EPI baked into the graphs
   bool items_dirty = true;
   int items_proposal = -1;  // proposal mode the work list and block shape were built for
+  std::vector<smcx_sched> items_sched;  // and the schedule of every replica
   int last_grid = 0;
   bool last_graph = false;
   // fluctuation accumulation: per-replica descriptors, (replica, tile) items, counts
@@ -75,6 +76,7 @@ void check_batch(const smcx_batch* b) {
 }
 
 void rebuild_items(smcx_batch* b) {
+  b->items_dirty = true;  // until the plan is whole: a refused one is made again
   std::vector<int2> items;
   int nq = 0, max_L = 0;
   for (size_t r = 0; r < b->lat.size(); r++) {
@@ -119,9 +121,23 @@ void rebuild_items(smcx_batch* b) {
   b->slots = slots;
   b->max_L = max_L;
   b->items_proposal = b->lat[0]->proposal;
+  b->items_sched.clear();
+  for (const smcx_lattice* h : b->lat) b->items_sched.push_back(h->sched);
   for (auto& g : b->graphs) cudaGraphExecDestroy(g.second);
   b->graphs.clear();
   b->items_dirty = false;
+}
+
+// The work list, the block shape, the room for directions and the captured graphs hold
+// for the schedules they were made for.  smcx_set_schedule and smcx_autotune act on a
+// replica, which does not know of its batch: compared on every call.
+bool plan_holds(const smcx_batch* b) {
+  if (b->items_dirty || b->items_proposal != b->lat[0]->proposal || b->items_sched.size() != b->lat.size()) return false;
+  for (size_t r = 0; r < b->lat.size(); r++) {
+    const smcx_sched &s = b->lat[r]->sched, &t = b->items_sched[r];
+    if (s.L != t.L || s.nt[0] != t.nt[0] || s.nt[1] != t.nt[1] || s.nt[2] != t.nt[2]) return false;
+  }
+  return true;
 }
 
 using bccfast::BatchKernelFn;
@@ -164,7 +180,7 @@ void batch_sweep(smcx_batch* b, const double* T, int64_t n_sweeps, uint64_t seed
 }
 
 static void batch_sweep_launch(smcx_batch* b, const double* T, int64_t n_sweeps, uint64_t seed) {
-  if (b->items_dirty || b->items_proposal != b->lat[0]->proposal) rebuild_items(b);
+  if (!plan_holds(b)) rebuild_items(b);
   const size_t R = b->lat.size();
   std::vector<bccfast::LatDesc> desc(R);
   int max_nA = 0;

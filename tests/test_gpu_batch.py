@@ -188,6 +188,61 @@ def test_batch_proposal_modes_in_turn(stream):
         l.close()
 
 
+@pytest.mark.parametrize("proposal", [smcx.PROPOSAL_SITE, smcx.PROPOSAL_TILE, smcx.PROPOSAL_BLOCK])
+def test_batch_follows_replica_schedules(stream, proposal):
+    """Schedules of single replicas change between the sweeps of a batch, by
+    smcx_set_schedule and smcx_autotune: longer link cells in the same tiles
+    (more phase directions), more and fewer tiles, 3^3 to 5^3 link-cell slots,
+    a schedule that batches refuse, and the first one again.  The sweep count
+    and the temperatures stay, so a captured graph would be replayed."""
+    dims = [(24, 26, 28), (40, 20, 36), (16, 40, 24)]
+    V = epi_gaussian(4, 4, 20.0, 41)
+    T = log_temperatures(len(dims), 500.0, 2500.0)
+    first = (3, (4, 4, 4))
+    lats = [_make(d, r, V, stream, first) for r, d in enumerate(dims)]
+    for l in lats:
+        l.set_proposal(proposal)
+    b = smcx.Batch(lats, stream)
+    cfg = [O.init_config(O.BCC, d, 4, [0.25] * 4, 100 + r) for r, d in enumerate(dims)]
+    stats = [np.zeros(4, np.int64) for _ in dims]
+    n = 0
+
+    def sweep_and_compare(what):
+        nonlocal n
+        b.sweep(T, 1, 43)
+        for r, d in enumerate(dims):
+            L, nt = lats[r].schedule()
+            stats[r] += O.sweep(O.BCC, d, 4, 4, V, cfg[r], T[r], 1, 43, sweep0=n, replica=r, L=L, nt=nt,
+                                proposal=proposal)
+            assert (lats[r].get_config() == cfg[r]).all(), f"replica {r}: {what}"
+            assert lats[r].state()[1].tolist() == stats[r].tolist(), f"replica {r}: {what}"
+        n += 1
+
+    sweep_and_compare("first")
+    for r, sched in [(1, (4, (4, 4, 4))), (1, (5, (4, 4, 4))), (0, (6, (4, 4, 4))),  # longer link cells
+                     (2, (3, (4, 8, 6))), (0, (3, (6, 6, 6))),                      # more tiles
+                     (2, (3, (2, 4, 2))), (1, (4, (2, 2, 2))),                      # fewer tiles, 5^3 slots
+                     (0, (8, (2, 2, 2))), (1, (10, (2, 2, 2)))]:
+        lats[r].set_schedule(sched)
+        sweep_and_compare(f"replica {r} to {sched}")
+    kept = lats[1].schedule()
+    lats[1].set_schedule((3, (2, 2, 2)))  # 7^3 slots: refused by batches
+    with pytest.raises(smcx.SmcxError) as e:
+        b.sweep(T, 1, 43)
+    assert e.value.code == smcx.E_UNSUPPORTED
+    lats[1].set_schedule(kept)
+    sweep_and_compare("the last plan after a refused one")
+    for l in lats:
+        l.set_schedule(first)
+    sweep_and_compare("first again")
+    lats[0].autotune(T[0], 1)
+    lats[2].set_schedule(None)
+    sweep_and_compare("tuned and library schedules")
+    b.close()
+    for l in lats:
+        l.close()
+
+
 def test_batch_mixed_proposal_modes_refused(stream):
     V = epi_gaussian(4, 4, 20.0, 1)
     dims = [(12, 12, 12), (16, 16, 16)]
