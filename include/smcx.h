@@ -231,8 +231,10 @@ int smcx_set_replica(smcx_lattice* h, int replica);
 #define SMCX_PROPOSAL_BLOCK 2
 int smcx_set_proposal(smcx_lattice* h, int mode);
 
-/* Threads per CTA of the BCC shared-memory kernel (0 = one thread per
- * link-cell slot; else a multiple of 32 up to 512).  Performance only. */
+/* Threads per CTA of the BCC shared-memory kernel (0 = the library's choice:
+ * several lanes per trial on lattices of few small tiles, else the fewest
+ * threads that cover the link-cell slots; otherwise a multiple of 32 up to
+ * 512).  Performance only. */
 int smcx_set_block(smcx_lattice* h, int threads);
 
 /* Replace the schedule (NULL = library's choice).  The trajectory depends on
@@ -406,14 +408,18 @@ int smcx_threshold_tables(double T, uint32_t* A, int* nA, uint32_t* B);
  *                       the tiles of its replica that come before it.
  *   smcx_batch_autotune times `trial_sweeps` batched sweeps for every
  *                       candidate (link cell 3 or 4, tiles of at most 12-20
- *                       cells, 128- or 256-thread CTAs) on snapshots of the
+ *                       cells, block sizes 0, 128 and 256 as in
+ *                       smcx_batch_set_block) on snapshots of the
  *                       configurations, restores them, and installs the
  *                       fastest candidate's schedules (read them back with
  *                       smcx_get_schedule) and block size (*threads).
  *   smcx_batch_energy   E[R], one smcx_energy per replica.
  *   smcx_batch_info     grid size, threads per CTA and whether the last call
  *                       replayed a graph.
- *   smcx_batch_set_block threads per CTA of the next sweeps: 0 (the fewest
+ *   smcx_batch_set_block threads per CTA of the next sweeps: 0 (the library's
+ *                       choice: 128 threads with four of them per trial while
+ *                       a colour has at most two tiles per SM, of at most 3^3
+ *                       link cells each; else the fewest
  *                       128-thread-or-smaller CTAs that cover a tile's link
  *                       cells with at most 2 slots per thread; 256 threads for
  *                       tiles of more than 128 link cells under a

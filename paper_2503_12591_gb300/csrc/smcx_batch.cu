@@ -75,16 +75,49 @@ void check_batch(const smcx_batch* b) {
   if (h0->shells.K != 4) fail(SMCX_E_UNSUPPORTED, "batched sweeps run 4-shell EPI tables");
 }
 
+// Threads per CTA and slots per thread for the replicas' schedules; `block` as set by
+// the caller (0: the library's choice).
+struct BlockShape {
+  int threads = 0, slots = 1;
+  bool group = false;
+};
+BlockShape block_shape(const smcx_batch* b, int block) {
+  BlockShape s;
+  int nq = 0, max_L = 0;
+  long long n_items = 0;
+  for (const smcx_lattice* h : b->lat) {
+    max_L = std::max(max_L, (int)h->sched.L);
+    n_items += (long long)(h->sched.nt[0] / 2) * (h->sched.nt[1] / 2) * (h->sched.nt[2] / 2);
+    nq = std::max(nq, bcc_slots_per_axis(h->n, h->sched));
+  }
+  // shared-direction proposals run one slot per thread: tiles of more than
+  // 128 slots take 256-thread CTAs unless 128 threads were asked for
+  const bool dir = b->lat[0]->proposal != 0;
+  if (block == 256 || (dir && block != 128 && nq * nq * nq > 128)) {
+    s.threads = 256;  // one slot per thread
+    if (nq * nq * nq > 256) fail(SMCX_E_UNSUPPORTED, "256-thread CTAs take tiles of at most 256 link-cell slots");
+  } else {
+    bcc_block_shape(nq, block, &s.threads, &s.slots);
+  }
+  if (s.slots > 2) fail(SMCX_E_UNSUPPORTED, "batched tiles need at most 256 link-cell slots");
+  // Four lanes per trial while a colour has at most two tiles per SM and no tile has
+  // more than 3^3 slots: 216 tiles 0.443 -> 0.362 ms a sweep, 343 tiles 0.894 -> 0.907.
+  // A block size that was set is kept.
+  s.group = block == 0 && nq <= 3 && n_items <= 2 * kSMs && (!dir || max_L <= 6);
+  if (s.group) s.threads = bccfast::kGroupThreads;
+  return s;
+}
+
 void rebuild_items(smcx_batch* b) {
   b->items_dirty = true;  // until the plan is whole: a refused one is made again
+  const BlockShape shape = block_shape(b, b->block);
   std::vector<int2> items;
-  int nq = 0, max_L = 0;
+  b->max_L = 0;
   for (size_t r = 0; r < b->lat.size(); r++) {
     const smcx_lattice* h = b->lat[r];
-    max_L = std::max(max_L, (int)h->sched.L);
+    b->max_L = std::max(b->max_L, (int)h->sched.L);
     const int per_colour = (h->sched.nt[0] / 2) * (h->sched.nt[1] / 2) * (h->sched.nt[2] / 2);
     for (int j = 0; j < per_colour; j++) items.push_back(make_int2((int)r, j));
-    nq = std::max(nq, bcc_slots_per_axis(h->n, h->sched));
   }
   // largest replicas first, so the tail of each colour pass holds small tiles
   std::stable_sort(items.begin(), items.end(), [&](const int2& a, const int2& c) {
@@ -101,25 +134,9 @@ void rebuild_items(smcx_batch* b) {
              "batch work list upload");
   check_cuda(cudaStreamSynchronize(b->stream), "batch work list sync");
   b->n_items = (int)items.size();
-  int threads, slots;
-  // shared-direction proposals run one slot per thread: tiles of more than
-  // 128 slots take 256-thread CTAs unless 128 threads were asked for
-  const bool dir = b->lat[0]->proposal != 0;
-  if (b->block == 256 || (dir && b->block != 128 && nq * nq * nq > 128)) {
-    threads = 256;  // one slot per thread
-    slots = 1;
-    if (nq * nq * nq > 256) fail(SMCX_E_UNSUPPORTED, "256-thread CTAs take tiles of at most 256 link-cell slots");
-  } else {
-    bcc_block_shape(nq, b->block, &threads, &slots);
-  }
-  if (slots > 2) fail(SMCX_E_UNSUPPORTED, "batched tiles need at most 256 link-cell slots");
-  // Four lanes per trial while a colour has at most two tiles per SM and no tile has
-  // more than 3^3 slots: 216 tiles 0.443 -> 0.362 ms a sweep, 343 tiles 0.894 -> 0.907.
-  // A block size that was set is kept.
-  b->group = b->block == 0 && nq <= 3 && b->n_items <= 2 * kSMs && (!dir || max_L <= 6);
-  b->threads = b->group ? bccfast::kGroupThreads : threads;
-  b->slots = slots;
-  b->max_L = max_L;
+  b->threads = shape.threads;
+  b->slots = shape.slots;
+  b->group = shape.group;
   b->items_proposal = b->lat[0]->proposal;
   b->items_sched.clear();
   for (const smcx_lattice* h : b->lat) b->items_sched.push_back(h->sched);
@@ -299,8 +316,8 @@ void batch_release(smcx_batch* b) {
   cudaFree(b->d_status);
 }
 
-// Autotuner: for each candidate (link cell L, tile target, threads per CTA)
-// assign every replica the schedule the candidate implies, time `trial`
+// Autotuner: for each candidate (link cell L, tile target, threads per CTA, 0 for the
+// library's choice) assign every replica the schedule the candidate implies, time `trial`
 // batched sweeps on a copy of the configurations, restore them, and keep the
 // fastest candidate.  The schedule defines the trajectory, so the choice is
 // reported (smcx_get_schedule on each replica) and a run can be reproduced.
@@ -332,10 +349,13 @@ void batch_autotune(smcx_batch* b, const double* T, int trial, int* best_threads
   std::vector<Cand> cands;
   // a tile pass takes 2 L^3 phase steps whatever the tile's size, so the
   // candidates trade tile size (lanes busy per step) against the number of
-  // items per colour (CTA rounds); shapes a kernel does not take are skipped
+  // items per colour (CTA rounds); shapes a kernel does not take are skipped.
+  // The library's own block shape is among them: several lanes per trial come
+  // with no set size (40 replicas of 18^3 cells, L = 3: 0.319 ms a sweep, 0.375 and
+  // 0.347 with 128 and 256 threads; 290 replicas 0.386, 0.386 and 0.366).
   for (int L : {3, 4})
     for (int target : {12, 13, 14, 15, 16, 17, 18, 20})
-      for (int th : {128, 256}) cands.push_back({L, target, th});
+      for (int th : {128, 256, 0}) cands.push_back({L, target, th});
   double best = 1e300;
   Cand bestc = cands[0];
   std::vector<smcx_sched> best_sched(R);
@@ -363,6 +383,10 @@ void batch_autotune(smcx_batch* b, const double* T, int trial, int* best_threads
     for (size_t r = 0; r < R; r++) usable = usable && bcc_fast_usable(b->lat[r], 256);
     if (!usable) continue;
     try {
+      if (c.threads == 0) {
+        const BlockShape own = block_shape(b, 0);
+        if (!own.group && own.threads >= 128) continue;  // one of the two before
+      }
       batch_sweep(b, T, 1, 0x5eedull);  // warm-up: instantiate, load tables
       check_cuda(cudaEventRecord(e0, b->stream), "event");
       batch_sweep(b, T, trial, 0x5eedull);

@@ -276,6 +276,29 @@ def test_batch_autotune_then_oracle(stream):
     b.close()
 
 
+def test_batch_autotune_finds_lanes_per_trial(stream):
+    """Few tiles of 3^3 slots: the library's own block shape (four lanes per
+    trial, 0.319 ms a sweep against 0.347 with 256 threads) is among the
+    candidates, wins, and stays in use afterwards."""
+    V = epi_gaussian(4, 4, 20.0, 2)
+    dims = [(18, 18, 18)] * 40
+    T = log_temperatures(len(dims), 500.0, 2500.0)
+    lats = [_make(d, r, V, stream, _sched(d)) for r, d in enumerate(dims)]
+    b = smcx.Batch(lats, stream)
+    b.set_block(256)
+    assert b.autotune(T, trial_sweeps=48) == 0
+    b.sweep(T, 3, 11)
+    assert b.info()["threads"] == 128
+    for r in (0, 17, 39):
+        L, nt = lats[r].schedule()
+        ref = O.init_config(O.BCC, dims[r], 4, [0.25] * 4, 100 + r)
+        O.sweep(O.BCC, dims[r], 4, 4, V, ref, T[r], 3, 11, replica=r, L=L, nt=nt)
+        assert (lats[r].get_config() == ref).all(), f"replica {r} schedule {(L, nt)}"
+    b.close()
+    for l in lats:
+        l.close()
+
+
 def test_batch_barrier_timeout_reports_and_recovers(stream):
     """A CTA that never arrives at the grid barrier: the other CTAs give up
     after the time limit, the call returns SMCX_E_TIMEOUT, and the context
