@@ -98,6 +98,32 @@ def test_cluster_labels_repeatable(stream):
     lat.close()
 
 
+def test_cluster_summary_limits(stream):
+    """The list of large clusters has room for N / min_size of them, the marks
+    and counts for max_out: from every cluster to none, one and all returned,
+    on one handle and (its first call) on another."""
+    kind, K, dims, M = smcx.BCC, 4, (24, 22, 20), 4
+    lat, V = _lattice(stream, kind, K, dims, M, smcx.INT8)
+    cfg = lat.get_config()
+    N = cfg.size
+    thr = int(np.quantile(O.local_energy2(kind, dims, M, K, V, cfg), 0.2))
+    olab, onc = O.clusters(kind, dims, M, K, V, cfg, thr)
+    lab = torch.empty(N, dtype=torch.int32, device="cuda")
+    assert lat.clusters(thr, lab.data_ptr()) == onc
+    largest = int(O.cluster_summary(olab, cfg, M, 1)[1][0])
+    for min_size in (N + 1, N, largest + 1, largest, N // 2, 40, 2, 1):
+        other, _ = _lattice(stream, kind, K, dims, M, smcx.INT8)
+        oroots, osizes, ocounts = O.cluster_summary(olab, cfg, M, min_size)
+        for most in (1, 50, N):
+            for h in (lat, other):
+                roots, sizes, counts = h.cluster_summary(lab.data_ptr(), min_size, most)
+                assert roots.tolist() == oroots[:most].tolist()
+                assert sizes.tolist() == osizes[:most].tolist()
+                assert counts.tolist() == ocounts[:most].tolist()
+        other.close()
+    lat.close()
+
+
 def test_cluster_errors(stream):
     lat = smcx.Lattice(smcx.BCC, (8, 8, 8), 4, [0.25] * 4, stream=stream)
     buf = torch.empty(lat.N, dtype=torch.int32, device="cuda")
