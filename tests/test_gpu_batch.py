@@ -299,21 +299,37 @@ def test_batch_autotune_finds_lanes_per_trial(stream):
         l.close()
 
 
-def test_batch_barrier_timeout_reports_and_recovers(stream):
-    """A CTA that never arrives at the grid barrier: the other CTAs give up
-    after the time limit, the call returns SMCX_E_TIMEOUT, and the context
-    keeps working."""
+@pytest.mark.parametrize("block,threads", [(0, 128), (256, 256)])
+def test_batch_wait_timeout_reports_and_recovers(stream, block, threads):
+    """A CTA that never reports its first tile pass: the passes that wait for
+    it give up after the time limit, the call returns SMCX_E_TIMEOUT and the
+    sweep counters stay.  From restored configurations the next sweeps are
+    right, on the kernel with four lanes per trial (block size 0, tiles of
+    3^3 slots) and on the one with a lane per trial."""
     V = epi_gaussian(4, 4, 20.0, 3)
-    lats = [_make(d, r, V, stream, _sched(d)) for r, d in enumerate(DIMS[:3])]
+    dims = [(12, 12, 12), (18, 14, 16), (13, 16, 18)]
+    T = [900.0, 1000.0, 1100.0]
+    scheds = [_sched(d, L=3, target=9) for d in dims]
+    lats = [_make(d, r, V, stream, scheds[r]) for r, d in enumerate(dims)]
+    cfg = [l.get_config().copy() for l in lats]
     b = smcx.Batch(lats, stream)
+    b.set_block(block)
     b.set_fault(0, 200)
     with pytest.raises(smcx.SmcxError) as e:
-        b.sweep([1000.0] * 3, 2, 1)
+        b.sweep(T, 2, 1)
     assert e.value.code == smcx.E_TIMEOUT
+    assert b.info()["threads"] == threads
     b.set_fault(-1, 2000)
-    b.sweep([1000.0] * 3, 1, 1)
-    torch.cuda.synchronize()
-    assert lats[0].energy() == lats[0].energy()
+    for l, c in zip(lats, cfg):
+        assert l.state()[0] == 0
+        l.set_config(c)
+    for n in (0, 2):
+        b.sweep(T, 2, 1)
+        assert b.info()["threads"] == threads
+        for r, d in enumerate(dims):
+            O.sweep(O.BCC, d, 4, 4, V, cfg[r], T[r], 2, 1, sweep0=n, replica=r, L=scheds[r][0], nt=scheds[r][1])
+            assert (lats[r].get_config() == cfg[r]).all(), f"replica {r}"
+    assert b.energy().tolist() == [O.energy(O.BCC, d, 4, 4, V, c) for d, c in zip(dims, cfg)]
     b.close()
 
 
