@@ -29,7 +29,7 @@ __host__ __device__ constexpr size_t progress_bytes(size_t replicas) { return 8 
 // first by their own index, the rest from a counter as they get done.  A pass waits
 // only for its own replica: until all tiles of that replica's previous colour are done.
 // They stand earlier in the list, so some CTA is at work on them or done, and the
-// entry furthest ahead never waits.  A wait lasts at most `timeout_ns`; a CTA that
+// first unfinished entry never waits.  A wait lasts at most `timeout_ns`; a CTA that
 // gives up sets the status, and all others stop when they see it.
 // Thread 0 publishes, draws and waits: a CTA barrier and a fence come between the
 // pass's writes and the counter, and between the counter and the next pass's reads.

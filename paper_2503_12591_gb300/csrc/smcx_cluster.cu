@@ -643,7 +643,7 @@ bccfast::LatDesc tile_desc(const smcx_lattice* hd, int edge, int* grid) {
     }
     if (g > 0x7FFFFFFFll) fail(SMCX_E_UNSUPPORTED, "lattice too large for the tile kernels");
     *grid = (int)g;
-    if (g >= 304) break;
+    if (g >= 2 * kSMs) break;
   }
   return D;
 }

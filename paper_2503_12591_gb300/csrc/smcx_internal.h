@@ -22,7 +22,9 @@ constexpr int kFCC = SMCX_FCC;
 constexpr int kMaxShells = 4;     // BCC 1..4, FCC 1..3
 constexpr int kMaxVec = 64;       // neighbour vectors of all shells in use
 constexpr int kMaxZ1 = 12;        // shell-1 size (BCC 8, FCC 12)
-constexpr int kSMs = 152;  // streaming multiprocessors
+// Streaming multiprocessors of a GB300, where the rules by tiles per SM were measured
+// (a choice among kernels of equal results; grids ask the device).
+constexpr int kSMs = 152;
 constexpr int kMaxSweepM = 8;     // species supported by the sweep kernels
 constexpr double kBoltzmannMeV = 8.617333262e-2;  // k_B in meV/K (exact SI)
 

@@ -171,7 +171,7 @@ bool fcc_reduce_usable(const smcx_lattice* hd, int nt[3]) {
       if (hd->n[a] < 2) return false;
       nt[a] = (hd->n[a] + edge - 1) / edge;
     }
-    if ((long long)nt[0] * nt[1] * nt[2] >= 304) break;
+    if ((long long)nt[0] * nt[1] * nt[2] >= 2 * kSMs) break;
   }
   return (long long)nt[0] * nt[1] * nt[2] < (1ll << 31);
 }

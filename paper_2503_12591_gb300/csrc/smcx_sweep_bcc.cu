@@ -160,8 +160,13 @@ void sweep_bcc_fast(smcx_lattice* hd, int nA, uint64_t seed, int64_t n_sweeps, i
   }
   // Several lanes per trial while the colour's tiles leave the GPU mostly idle: 3^3 slots
   // up to two tiles per SM (216 tiles 0.443 -> 0.362 ms, 343 tiles 0.894 -> 0.907), 4^3
-  // slots up to one (125 tiles, L = 3 0.443 -> 0.394 ms, 216 tiles 0.469 -> 0.504).  A
-  // block size that was set is kept.
+  // slots up to one (125 tiles, L = 3 0.443 -> 0.394 ms, 216 tiles 0.469 -> 0.504).
+  // Below these lines every form gains against a lane per trial: 2, 3 and 4 shells, one
+  // and two counter words, two and three planes, shared directions, 1^3 to 4^3 slots, L =
+  // 3 and 4, 1 to 294 tiles (1 to 150 of 4^3 slots), 1.03 to 1.76 times as fast.  Least:
+  // 2 shells with 2^3 slots (294 tiles, L = 3 0.345 -> 0.332 ms) and seven species with
+  // three planes (3^3 slots, 294 tiles, L = 4 1.165 -> 1.132).  A block size that was set
+  // is kept.
   const int tiles = (sc.nt[0] / 2) * (sc.nt[1] / 2) * (sc.nt[2] / 2);
   if (hd->bcc_threads == 0 && D.NQ <= bccfast::kMaxGroupNQ && tiles <= (D.NQ <= 3 ? 2 : 1) * kSMs &&
       (D.proposal == 0 || D.L <= 6))
