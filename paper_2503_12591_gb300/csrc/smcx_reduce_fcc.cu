@@ -159,21 +159,15 @@ __global__ void __launch_bounds__(256, 4) k_fcc_qsro_energy(const LatDesc D, con
 
 }  // namespace fccfast
 
-// Tiles for a reduction over an FCC lattice of at most eight species: of at most
-// 15 cells, smaller ones (down to 4 cells) until there are two per SM, edges of 2
+// Tiles for a reduction over an FCC lattice of at most eight species: edges of 2
 // cells at least (the staging wraps a coordinate once) and a store whose cells
 // can be read as words.
 bool fcc_reduce_usable(const smcx_lattice* hd, int nt[3]) {
   if (hd->kind != kFCC || hd->M > kMaxSweepM || !hd->have_epi || hd->shells.K > 3) return false;
   if (hd->kernel_choice == SMCX_KERNEL_GENERIC || reinterpret_cast<uintptr_t>(hd->d_sites) % 4 != 0) return false;
-  for (int edge : {fccfast::TMAX, 12, 10, 8, 6, 4}) {
-    for (int a = 0; a < 3; a++) {
-      if (hd->n[a] < 2) return false;
-      nt[a] = (hd->n[a] + edge - 1) / edge;
-    }
-    if ((long long)nt[0] * nt[1] * nt[2] >= 2 * kSMs) break;
-  }
-  return (long long)nt[0] * nt[1] * nt[2] < (1ll << 31);
+  for (int a = 0; a < 3; a++)
+    if (hd->n[a] < 2) return false;
+  return bccfast::reduction_tiles(hd->n, fccfast::TMAX, nt) < (1ll << 31);
 }
 
 static bccfast::LatDesc reduce_desc(const smcx_lattice* hd, const int nt[3]) {

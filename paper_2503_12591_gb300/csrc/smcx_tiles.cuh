@@ -43,6 +43,27 @@ struct CellIndex {
   }
 };
 
+// Tile counts nt of a reduction that stages each tile with its 2-cell halo, and the
+// number of tiles.  Lattices of at least two tiles per SM take the largest tiles, of
+// `most` or 12 cells.  Smaller ones take the largest edge that gives 100 tiles: below
+// that SMs idle, above it the halo costs more than the SMs gain.  Wall time of FCC pair
+// counts against tiles for two per SM throughout: 44^3 cells, 4 species, 2 shells 42 -> 30
+// us, 36^3, 8 species, 3 shells 58 -> 36; local energies of 36^3 BCC cells, 4 shells 16
+// -> 8 us.  (Gathers from global memory take 32, 47 and 18.)
+inline long long reduction_tiles(const int n[3], int most, int nt[3]) {
+  auto tiles = [&](int edge) {
+    long long g = 1;
+    for (int a = 0; a < 3; a++) g *= nt[a] = (n[a] + edge - 1) / edge;
+    return g;
+  };
+  long long g = 0;
+  for (int edge : {most, 12})
+    if ((g = tiles(edge)) >= 2 * kSMs) return g;
+  for (int edge : {12, 10, 8, 7, 6})
+    if ((g = tiles(edge)) >= 100) return g;
+  return tiles(4);
+}
+
 // acc += x * one (one: 0 or 1), without the branch that the compiler makes of a test of
 // the lane's species: where lanes differ, it runs every branch in turn.
 __device__ __forceinline__ void add_if(uint32_t& acc, uint32_t x, uint32_t one) {

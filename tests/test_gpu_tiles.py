@@ -225,3 +225,19 @@ def test_shared_directions_of_long_link_cells(kind, L, nt, dims, proposal):
         b.close()
         lat2.close()
     lat.close()
+
+
+@pytest.mark.parametrize("dims", [(25, 24, 27), (28, 29, 27), (32, 31, 33), (40, 39, 36), (48, 50, 41), (60, 49, 55), (7, 150, 31)])
+@pytest.mark.parametrize("kind,M,K,storage", [(smcx.FCC, 5, 3, smcx.PACKED4), (smcx.FCC, 8, 2, smcx.INT8),
+                                              (smcx.BCC, 4, 4, smcx.PACKED4), (smcx.BCC, 3, 2, smcx.INT8)])
+def test_reduction_tile_edges(dims, kind, M, K, storage):
+    # lattices of fewer than two 12-cell tiles per SM: tiles of 4, 6, 7, 8, 10 and 12 cells;
+    # two-shell BCC int8 lattices on both sides of the 2^16 sites up to which they gather
+    lat, cfg, V = _lattice(kind, dims, M, K, storage, 43)
+    assert (lat.pair_counts() == O.pair_counts(kind, dims, M, K, cfg)).all()
+    assert lat.energy() == O.energy(kind, dims, M, K, V, cfg)
+    e2 = torch.empty(cfg.size, dtype=torch.int32, device="cuda")
+    lat.local_energy(e2.data_ptr())
+    lat.synchronize()
+    assert (e2.cpu().numpy() == O.local_energy2(kind, dims, M, K, V, cfg)).all()
+    lat.close()
