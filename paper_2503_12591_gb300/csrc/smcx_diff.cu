@@ -118,7 +118,7 @@ __host__ __device__ constexpr HalfVecs make_half_vecs() {
 // after 20 sites at most (20 x 12 < 256).  Bound by issue; 4096 configurations of
 // 1,024 sites take 54 us against 215 for k_pair_counts_batch, which makes one
 // shared atomic per neighbour over whole shells (50 a site) and stays for more
-// than eight species and for edges of one cell.
+// than eight species, for edges of one cell and where whole_shells says so.
 template <int KIND, int K, int W>
 __global__ void __launch_bounds__(256) k_pair_counts_batch_half(const int8_t* __restrict__ cfg, long long B, int nx,
                                                                 int ny, int nz, int M, long long* __restrict__ out) {
@@ -236,6 +236,24 @@ __global__ void __launch_bounds__(256) k_pair_counts_batch_half(const int8_t* __
     }
     __syncthreads();
   }
+}
+
+// Five to eight species on BCC lattices of at most three shells: few neighbours against
+// the 16 K accumulators that every warp empties per configuration, so one shared
+// atomic per neighbour is the faster on small configurations and small batches.  us,
+// atomics and half shells, 4096 configurations of eight species: 3 shells, 3^3 cells 21
+// and 19, 4^3 27 and 29, 5^3 37 and 49, 6^3 57 and 90, 7^3 84 and 115, 8^3 115 and 117, 9^3
+// 162 and 147; 2 shells, 5^3 29 and 27, 6^3 39 and 45, 7^3 55 and 58, 8^3 72 and 62; one
+// shell, 5^3 21 and 19, 6^3 25 and 31, 7^3 35 and 41, 8^3 44 and 45.  600 configurations of
+// 2^3 to 4^3 cells 6.2 and 8.2; 64 of up to 8^3 6.2 to 8.3 and 8.2 to 10.3.  One shell,
+// 20^3 cells: 64 configurations 37 and 51, 200 51 and 57, 600 88 and 80.  With four shells
+// half shells are the faster (4096 of 6^3 122 and 115, of 8^3 217 and 143).
+bool whole_shells(int kind, int M, int K, int ncell, long long B) {
+  if (kind != kBCC || M <= 4 || K == 4) return false;
+  if (B <= kSMs && ncell < 600) return true;
+  if (B <= 2 * kSMs && (K == 1 || ncell < 450)) return true;
+  if (B <= 4 * kSMs && ncell < 150) return true;
+  return K == 3 ? ncell >= 60 && ncell < 450 : ncell >= 150 && ncell < (K == 2 ? 300 : 450);
 }
 
 // E_b = 1/2 sum_i V_i C_bi (FP64 sum, FP32 result): one warp per config.
@@ -395,8 +413,8 @@ int smcx_pair_counts_batch(int kind, int nx, int ny, int nz, int M, int K, const
     const int grid = (int)std::min<long long>(B, 65535);
     // at most eight species: counted in registers over half shells (edges of the
     // reach of 2 cells at least, so that one wrap covers every displacement)
-    if (M <= 8 && nx >= 2 && ny >= 2 && nz >= 2) {
-      const int ncell = nx * ny * nz;
+    const int ncell = nx * ny * nz;
+    if (M <= 8 && nx >= 2 && ny >= 2 && nz >= 2 && !whole_shells(kind, M, K, ncell, B)) {
       const int threads = std::min(256, (ncell + 31) / 32 * 32);
       const size_t sm = (size_t)(N + 3) / 4 * 4;
       auto run = [&](auto kern) {

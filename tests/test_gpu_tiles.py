@@ -89,6 +89,25 @@ def test_pair_counts_batch_sizes(kind, dims, M, K, B):
             assert (C[b] == O.pair_counts(kind, dims, M, K, cfg[b])).all()
 
 
+@pytest.mark.parametrize("dims,B", [((3, 4, 5), 3), ((3, 3, 5), 600), ((3, 3, 5), 620), ((5, 5, 5), 620), ((6, 5, 5), 310),
+                                    ((6, 7, 7), 310), ((7, 7, 7), 310), ((8, 8, 7), 310), ((8, 8, 8), 160), ((9, 8, 8), 5)])
+@pytest.mark.parametrize("M,K", [(5, 1), (8, 1), (8, 2), (5, 3), (8, 3), (6, 4)])
+def test_pair_counts_batch_many_species(dims, B, M, K):
+    # five to eight species: both sides of the sizes at which whole shells take over
+    # from half shells, aligned and not, one configuration with an id out of range
+    N = O.n_sites(smcx.BCC, dims)
+    cfg = np.random.default_rng(12).integers(0, M, (B, N)).astype(np.int8)
+    cfg[B - 1, N // 2] = M
+    pad = torch.zeros(B * N + 3, dtype=torch.int8, device="cuda")
+    for off in (0, 2):
+        view = pad[off:off + B * N]
+        view.copy_(torch.from_numpy(cfg.reshape(-1)))
+        C = diff.pair_counts(view.view(B, N), smcx.BCC, dims, M, K).cpu().numpy()
+        for b in [*range(0, B - 1, max(1, B // 8))]:
+            assert (C[b] == O.pair_counts(smcx.BCC, dims, M, K, cfg[b])).all()
+        assert (C[B - 1] == -1).all()
+
+
 @pytest.mark.parametrize("dims,nt", [((40, 38, 42), (12, 12, 12)), ((18, 21, 40), (2, 2, 2)), ((34, 33, 32), (2, 2, 2))])
 @pytest.mark.parametrize("M,K,storage", [(5, 3, smcx.PACKED4), (4, 2, smcx.INT8), (8, 3, smcx.INT8)])
 def test_qsro_sweeps_few_and_many_tiles(dims, nt, M, K, storage):
