@@ -255,9 +255,17 @@ static void batch_sweep_launch(smcx_batch* b, const double* T, int64_t n_sweeps,
   }
   int n_int = (int)n_sweeps;
   int max_nA_arg = nA_cap;
+  // Five to eight species (two counter words): every CTA keeps its tile while there is a
+  // CTA for each and the SMs are evenly filled.  4 replicas of 160^3 cells, six species
+  // (864 tiles, L = 3) 1.82 -> 1.65 ms a sweep, 22 of 84^3 (594) 1.26 -> 1.19, 92 of 80^3
+  // (736, L = 4) 3.23 -> 3.02; unevenly filled, 3 of 160^3 (648) 1.33 -> 1.43, 62 of 60^3
+  // (496) 1.19 -> 1.23.  With one word drawing is the faster for most counts (594 tiles
+  // 0.86 ms, in place 0.93).
+  const int rows = (b->n_items + nsm - 1) / nsm;
+  int in_place = !b->group && nw == 2 && grid == b->n_items && 25ll * b->n_items >= 23ll * rows * nsm;
   void* args[] = {(void*)&Q, (void*)&b->d_desc, (void*)&b->d_items, (void*)&b->n_items, (void*)&n_int,
                   (void*)&b->d_progress, (void*)&b->d_status, (void*)&b->timeout_ns, (void*)&b->skip_cta,
-                  (void*)&max_nA_arg};
+                  (void*)&in_place, (void*)&max_nA_arg};
   if (b->graph_V != b->lat[0]->V) {
     for (auto& g : b->graphs) cudaGraphExecDestroy(g.second);
     b->graphs.clear();

@@ -38,10 +38,11 @@ __host__ __device__ constexpr size_t progress_bytes(size_t replicas) { return 8 
 // with CTA b on the items b, b + G, ... of a colour and a grid barrier after it: the
 // last items of every colour left most SMs idle.  Drawn from a counter 4.55 ms; with
 // the next colour begun before this one ends 4.00 ms.
-template <class Pass>
+// KEEP: with in_place set (and a CTA per item) every CTA keeps its item, nothing is drawn.
+template <bool KEEP, class Pass>
 __device__ __forceinline__ void batch_loop(const LatDesc* __restrict__ descs, const int2* __restrict__ items,
                                            int n_items, int n_sweeps, Progress* pr, int* status,
-                                           long long timeout_ns, int skip_cta, Pass pass) {
+                                           long long timeout_ns, int skip_cta, int in_place, Pass pass) {
   __shared__ int s_item, s_epoch;  // item < 0: no more work
   unsigned long long base = 0;     // thread 0: list position of item 0 of this colour
   int item = blockIdx.x, epoch = 0;  // epoch: colours since the launch began
@@ -55,14 +56,20 @@ __device__ __forceinline__ void batch_loop(const LatDesc* __restrict__ descs, co
     if (threadIdx.x == 0) {
       __threadfence();
       atomicAdd(&pr->done[it.x], 1ull);
-      const unsigned long long g = atomicAdd(&pr->drawn, 1ull) + gridDim.x;
       int next = -1;
-      while (g - base >= (unsigned)n_items) {
-        base += (unsigned)n_items;
+      if (KEEP && in_place) {
+        next = item;
         epoch++;
-      }
-      if (epoch < n_epochs) {
+      } else {
+        const unsigned long long g = atomicAdd(&pr->drawn, 1ull) + gridDim.x;
+        while (g - base >= (unsigned)n_items) {
+          base += (unsigned)n_items;
+          epoch++;
+        }
         next = (int)(g - base);
+      }
+      if (epoch >= n_epochs) next = -1;
+      if (next >= 0) {
         const int r = items[next].x;
         const LatDesc& R = descs[r];
         const unsigned per_colour = (unsigned)((R.nt[0] / 2) * (R.nt[1] / 2) * (R.nt[2] / 2));
@@ -92,13 +99,13 @@ __device__ __forceinline__ void batch_loop(const LatDesc* __restrict__ descs, co
 template <int K, int NW, int PL, int SLOTS, int PROP>
 __device__ __forceinline__ void batch_body(const Planes& Q, const LatDesc* __restrict__ descs,
                                            const int2* __restrict__ items, int n_items, int n_sweeps, Progress* pr,
-                                           int* status, long long timeout_ns, int skip_cta, int max_nA) {
+                                           int* status, long long timeout_ns, int skip_cta, int in_place, int max_nA) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ unsigned long long s_stat[3];
   uint32_t* sA = reinterpret_cast<uint32_t*>(smem + 2 * SUB);
   uint32_t* sB = sA + max_nA;
   uint8_t* s_dir = reinterpret_cast<uint8_t*>(sB + kNB);
-  batch_loop(descs, items, n_items, n_sweeps, pr, status, timeout_ns, skip_cta,
+  batch_loop<(NW > 1)>(descs, items, n_items, n_sweeps, pr, status, timeout_ns, skip_cta, in_place,
              [&](const LatDesc& D, int tc, int jt, unsigned long long sweep) {
                bcc_tile_pass<K, NW, PL, SLOTS, PROP>(D, Q, tc, jt, sweep, smem, sA, sB, s_dir, s_stat);
              });
@@ -110,32 +117,37 @@ __device__ __forceinline__ void batch_body(const Planes& Q, const LatDesc* __res
 template <int K, int NW, int PL, int SLOTS, int PROP>
 __global__ void __launch_bounds__(128, 6)
     k_bcc_batch(const Planes Q, const LatDesc* __restrict__ descs, const int2* __restrict__ items, int n_items,
-                int n_sweeps, Progress* pr, int* status, long long timeout_ns, int skip_cta, int max_nA) {
-  batch_body<K, NW, PL, SLOTS, PROP>(Q, descs, items, n_items, n_sweeps, pr, status, timeout_ns, skip_cta, max_nA);
+                int n_sweeps, Progress* pr, int* status, long long timeout_ns, int skip_cta, int in_place,
+                int max_nA) {
+  batch_body<K, NW, PL, SLOTS, PROP>(Q, descs, items, n_items, n_sweeps, pr, status, timeout_ns, skip_cta, in_place,
+                             max_nA);
 }
 template <int K, int NW, int PL, int PROP>
 __global__ void __launch_bounds__(256, 3)
     k_bcc_batch256(const Planes Q, const LatDesc* __restrict__ descs, const int2* __restrict__ items, int n_items,
-                   int n_sweeps, Progress* pr, int* status, long long timeout_ns, int skip_cta, int max_nA) {
-  batch_body<K, NW, PL, 1, PROP>(Q, descs, items, n_items, n_sweeps, pr, status, timeout_ns, skip_cta, max_nA);
+                   int n_sweeps, Progress* pr, int* status, long long timeout_ns, int skip_cta, int in_place,
+                   int max_nA) {
+  batch_body<K, NW, PL, 1, PROP>(Q, descs, items, n_items, n_sweeps, pr, status, timeout_ns, skip_cta, in_place,
+                             max_nA);
 }
 
 // Several lanes per trial (smcx_bcc_group.cuh), for few tiles of at most 3^3 slots.
 template <int LN, int K, int NW, int PL>
 __global__ void __launch_bounds__(kGroupThreads, 4)
     k_bcc_batch_group(const Planes Q, const LatDesc* __restrict__ descs, const int2* __restrict__ items, int n_items,
-                      int n_sweeps, Progress* pr, int* status, long long timeout_ns, int skip_cta, int max_nA) {
+                      int n_sweeps, Progress* pr, int* status, long long timeout_ns, int skip_cta, int in_place,
+                      int max_nA) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ __align__(16) GroupMem M;
   uint32_t* sA = reinterpret_cast<uint32_t*>(smem + 2 * SUB);
-  batch_loop(descs, items, n_items, n_sweeps, pr, status, timeout_ns, skip_cta,
+  batch_loop<false>(descs, items, n_items, n_sweeps, pr, status, timeout_ns, skip_cta, in_place,
              [&](const LatDesc& D, int tc, int jt, unsigned long long sweep) {
                group_pass<LN, K, NW, PL>(D, Q, tc, jt, sweep, smem, sA, sA + max_nA, M);
              });
 }
 
 using BatchKernelFn = void (*)(const Planes, const LatDesc*, const int2*, int, int, Progress*, int*, long long, int,
-                               int);
+                               int, int);
 
 }  // namespace bccfast
 

@@ -157,6 +157,41 @@ def test_batch_list_longer_than_the_grid(proposal, R, lo, hi, tile):
     b.close()
 
 
+@pytest.mark.parametrize("M,R,block", [(6, 56, 0), (6, 57, 0), (8, 57, 256), (5, 19, 128), (6, 48, 0), (4, 57, 0)])
+def test_batch_tiles_in_place(M, R, block):
+    # 8 tiles a replica and colour: two counter words on evenly filled SMs (448, 456 and
+    # 152 tiles) keep their tiles, 384 tiles and one word draw them
+    stream = torch.cuda.current_stream()
+    V = epi_gaussian(4, M, 20.0, 7)
+
+    def lattice(r):
+        lat = smcx.Lattice(smcx.BCC, (24, 25 + r % 3, 26), M, [1.0 / M] * M, init_seed=70 + r, storage=smcx.INT8,
+                           sched=(3, (4, 4, 4)), stream=stream)
+        lat.set_replica(r)
+        lat.set_epi(V)
+        return lat
+
+    T = np.linspace(500.0, 2400.0, R)
+    lats = [lattice(r) for r in range(R)]
+    b = smcx.Batch(lats, stream)
+    b.set_block(block)
+    b.sweep(T, 1, 9)
+    b.sweep(T, 3, 9)
+    assert b.info()["grid"] == 8 * R
+    for r in range(0, R, 3):
+        one = lattice(r)
+        one.sweep(T[r], 4, 9)
+        assert (lats[r].get_config() == one.get_config()).all()
+        assert lats[r].state()[1].tolist() == one.state()[1].tolist()
+        one.close()
+    cfg = O.init_config(O.BCC, (24, 25, 26), M, [1.0 / M] * M, 70)
+    O.sweep(O.BCC, (24, 25, 26), M, 4, V, cfg, T[0], 4, 9, L=3, nt=(4, 4, 4))
+    assert (lats[0].get_config() == cfg).all()
+    b.close()
+    for lat in lats:
+        lat.close()
+
+
 @pytest.mark.parametrize("L,nt,dims", [(3, 2, (24, 23, 22)), (3, 2, (30, 27, 25)), (3, 2, (36, 33, 31)), (4, 2, (32, 27, 29)),
                                        (4, 2, (40, 33, 36)), (4, 4, (44, 43, 42)), (5, 2, (40, 34, 31)), (6, 2, (40, 38, 36))])
 @pytest.mark.parametrize("M,proposal,storage", [(4, 0, smcx.PACKED4), (4, 1, smcx.PACKED4), (4, 2, smcx.INT8), (6, 0, smcx.INT8)])
