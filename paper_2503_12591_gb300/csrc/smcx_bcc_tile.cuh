@@ -48,7 +48,10 @@ constexpr int BOX = 24;            // usable box edge (tile <= 20 with halo 2)
 // these orders 1.0 (5^3, L = 4), 1.14 (6^3, L = 3), 1.25 (5^3, L = 3), 1.5 (4^3, L = 4).
 // Sweeps of 400^3 cells, plain and ordered: 15-cell tiles L = 3 4.01 and 3.68 ms (shared
 // directions 2.69 and 2.33), 18-cell tiles L = 3 4.25 and 3.83 ms; 256^3 cells, 16-cell
-// tiles L = 4 1.37 and 1.21 ms.  Shapes outside the table gained less or nothing.
+// tiles L = 4 1.37 and 1.21 ms.  Shapes outside the table gained less or nothing.  Of
+// 6^3 slots whose last layer holds one cell (16-cell tiles, L = 3) whole warps of the
+// plain order idle in most phases: with two counter words and three or four shells they
+// stay in it (256^3 cells, six and eight species 2.04 and 2.38 ms, ordered 2.12 and 2.53).
 constexpr int kOrderMinNQ = 4, kOrderMaxNQ = 6, kOrderMinL = 3, kOrderMaxL = 5;
 __host__ __device__ constexpr int order_lanes(int nq) { return (nq * nq * nq + 31) / 32 * 32; }
 
@@ -565,7 +568,8 @@ __device__ __forceinline__ void bcc_tile_pass(const LatDesc& D, const Planes& Q,
   // load; passes with a direction per trial have no registers to hold it.
   const int NQ = D.NQ, L = D.L, n_dir = 2 * L * L * L;
   const bool ordered = NQ >= kOrderMinNQ && NQ <= kOrderMaxNQ && L >= kOrderMinL && L <= kOrderMaxL &&
-                       nth * SLOTS >= order_lanes(NQ);
+                       nth * SLOTS >= order_lanes(NQ) &&
+                       (NW == 1 || K == 2 || NQ < 6 || max(ts[0], max(ts[1], ts[2])) > L * (NQ - 1) + 1);
   auto slot_of = [&](int j) {
     const int t = tid + j * nth;
     if (!ordered) return t;

@@ -192,7 +192,8 @@ def test_batch_tiles_in_place(M, R, block):
         lat.close()
 
 
-@pytest.mark.parametrize("L,nt,dims", [(3, 2, (24, 23, 22)), (3, 2, (30, 27, 25)), (3, 2, (36, 33, 31)), (4, 2, (32, 27, 29)),
+@pytest.mark.parametrize("L,nt,dims", [(3, 2, (24, 23, 22)), (3, 2, (30, 27, 25)), (3, 2, (36, 33, 31)), (3, 2, (32, 31, 30)),
+                                       (4, 2, (32, 27, 29)),
                                        (4, 2, (40, 33, 36)), (4, 4, (44, 43, 42)), (5, 2, (40, 34, 31)), (6, 2, (40, 38, 36))])
 @pytest.mark.parametrize("M,proposal,storage", [(4, 0, smcx.PACKED4), (4, 1, smcx.PACKED4), (4, 2, smcx.INT8), (6, 0, smcx.INT8)])
 def test_bcc_lane_orders(L, nt, dims, M, proposal, storage):
