@@ -56,20 +56,16 @@ __device__ __forceinline__ void batch_loop(const LatDesc* __restrict__ descs, co
     if (threadIdx.x == 0) {
       __threadfence();
       atomicAdd(&pr->done[it.x], 1ull);
-      int next = -1;
-      if (KEEP && in_place) {
-        next = item;
-        epoch++;
-      } else {
+      auto draw = [&]() {
         const unsigned long long g = atomicAdd(&pr->drawn, 1ull) + gridDim.x;
         while (g - base >= (unsigned)n_items) {
           base += (unsigned)n_items;
           epoch++;
         }
-        next = (int)(g - base);
-      }
-      if (epoch >= n_epochs) next = -1;
-      if (next >= 0) {
+        return (int)(g - base);
+      };
+      // `next` once its replica's previous colour is done, -1 if the launch stops
+      auto wait = [&](int next) {
         const int r = items[next].x;
         const LatDesc& R = descs[r];
         const unsigned per_colour = (unsigned)((R.nt[0] / 2) * (R.nt[1] / 2) * (R.nt[2] / 2));
@@ -85,6 +81,22 @@ __device__ __forceinline__ void batch_loop(const LatDesc* __restrict__ descs, co
           __nanosleep(64);
         }
         __threadfence();
+        return next;
+      };
+      int next = -1;
+      if constexpr (KEEP) {
+        // two paths to `next` before the test of the epoch: fewer spills than one
+        if (in_place) {
+          next = item;
+          epoch++;
+        } else {
+          next = draw();
+        }
+        if (epoch >= n_epochs) next = -1;
+        if (next >= 0) next = wait(next);
+      } else {
+        const int drawn = draw();
+        if (epoch < n_epochs) next = wait(drawn);
       }
       s_item = next;
       s_epoch = epoch;
